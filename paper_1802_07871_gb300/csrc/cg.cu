@@ -389,12 +389,15 @@ void launch_block_setup(const DevState& S, cudaStream_t st) {
 }
 
 // y = M_b^-1 r for the warp's block: every lane of a full warp, i = 32b +
-// lane, r_i of this lane (zero where no atom).
+// lane, r_i of this lane (zero where no atom). A warp wholly past the last
+// atom (the tail of a 256-atom tile) has no block: binv ends at the last
+// started one, so such a warp reads nothing.
 // The block is stored row by row (row a = element (a, j) for j = 0..31,
 // contiguous), so a lane reads its row with 16-byte loads (4 in FP16, 16 in
 // FP64; the inverse is symmetric, so the row is also the column).
 template <class R>
-__device__ inline R block_apply(const typename BlockStore<R>::T* __restrict__ binv, int i, R ri) {
+__device__ inline R block_apply(const typename BlockStore<R>::T* __restrict__ binv, int N, int i, R ri) {
+  if ((i & ~31) >= N) return R(0);   // (uniform over the warp)
   using BT = typename BlockStore<R>::T;
   constexpr int NV = 32 * (int)sizeof(BT) / 16;
   const uint4* rp = reinterpret_cast<const uint4*>(binv + (size_t)(i >> 5) * 1024 + (size_t)(i & 31) * 32);
@@ -618,7 +621,7 @@ __global__ void __launch_bounds__(256)
   {
     // y = M^-1 r (the block product takes every lane of the warp)
     R ri = rid >= 0 ? r[i] : R(0);
-    R yi = binv ? block_apply(binv, i, ri) : (rid >= 0 ? dinv[i] * ri : R(0));
+    R yi = binv ? block_apply(binv, N, i, ri) : (rid >= 0 ? dinv[i] * ri : R(0));
     if (rid >= 0) {
       y[i] = yi;
       part[0] = yi;
@@ -770,7 +773,7 @@ __global__ void __launch_bounds__(256)
     }
     // y = M^-1 r: the block product takes every lane of the warp (blocks do
     // not couple replicas, so a converged replica's lanes enter with r = 0)
-    R yi = binv ? block_apply(binv, i, ri) : (act ? dinv[i] * ri : R(0));
+    R yi = binv ? block_apply(binv, N, i, ri) : (act ? dinv[i] * ri : R(0));
     if (act) {
       y[i] = yi;
       part[0] += yi;
