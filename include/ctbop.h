@@ -252,7 +252,8 @@ int ctbop_status(ctbop_system* s, ctbop_stats* st);
 /* 0 kick + drift, 1 neighbour lists (flag-guarded, no-op without a rebuild),
  * 2 bond orders (Eq. 2, 7), 3 charge-system assembly, 4 CG start, 5 CG matrix
  * pass, 6 CG update, 7 charges from the CG solution, 8 covalent force slots,
- * 9 charge forces + slot gather + half kick. */
+ * 9 charge forces + slot gather + half kick. Systems whose charge solve runs
+ * as one kernel (small and medium ones) report the whole solve under 5. */
 
 /* Run n_steps velocity-Verlet steps (same arithmetic as ctbop_step) with
  * every kernel launched directly and bracketed by CUDA events on the

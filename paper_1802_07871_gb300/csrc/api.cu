@@ -403,6 +403,9 @@ static int alloc_atoms(ctbop_system* s) {
   CK(dalloc(s->rep_buf, &S.cg_hist, 1));
   CK(dalloc(s->rep_buf, &S.cg_active, 1));
   CK(dalloc(s->rep_buf, &S.cg_total, 1));
+  CK(dalloc(s->rep_buf, &S.solve_ctl, 4));
+  CK(dalloc(s->rep_buf, &S.solve_part, (size_t)2 * 6 * SOLVE_MAX_BLOCKS));
+  CK(zero_async(s, S.solve_ctl, 4 * sizeof(int)));
   CK(zero_async(s, S.rep_acc, sizeof(double) * s->R * RA_STRIDE));
   CK(zero_async(s, S.rebuild_count, sizeof(long long)));
   CK(zero_async(s, S.err, sizeof(unsigned)));
@@ -465,6 +468,7 @@ static int alloc_lists(ctbop_system* s, int cap_cov, int cap_all) {
   }
   s->alloc_cov = cap_cov;
   s->alloc_all = cap_all;
+  CK(s->mixed ? plan_cg_solve<float>(S, s->off.data()) : plan_cg_solve<double>(S, s->off.data()));
   return CTBOP_OK;
 }
 
@@ -497,14 +501,32 @@ static void enqueue_middle(ctbop_system* s, const PotParams<Rr>& P, cudaStream_t
   launch_bond<Rr>(S, P, st);
   launch_assemble<Rr>(S, P, s->T, st);
   if (S.precond) launch_block_setup<Rr>(S, st);
-  launch_cg_begin<Rr>(S, s->T, st, cg_tol(s));
+  if (S.solver == SOLVE_LAUNCHES) launch_cg_begin<Rr>(S, s->T, st, cg_tol(s));
+}
+
+// The solve on what enqueue_middle prepared, by the host: one launch, or
+// iterations of two with the device's active flag polled every few.
+template <class Rr>
+static int solve_direct(ctbop_system* s, const SolveCfg& cfg, const double* rhs, cudaStream_t st) {
+  DevState& S = s->S;
+  if (S.solver != SOLVE_LAUNCHES) {
+    CK(launch_cg_solve<Rr>(S, s->T, cfg.tol, cfg.max_iter, rhs, st));
+    return CTBOP_OK;
+  }
+  for (int it = 0; it < cfg.max_iter + 4; it += 4) {
+    for (int k = 0; k < 4; ++k) launch_cg_iter<Rr>(S, cfg, st);
+    CK(cudaMemcpyAsync(s->h_int, S.cg_active, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    if (*s->h_int == 0) break;
+  }
+  return CTBOP_OK;
 }
 
 template <class Rr>
 static void enqueue_back(ctbop_system* s, const PotParams<Rr>& P, cudaStream_t st, bool md, double dt,
                          bool solve) {
   DevState& S = s->S;
-  if (solve) launch_cg_end<Rr>(S, st);
+  if (solve && S.solver == SOLVE_LAUNCHES) launch_cg_end<Rr>(S, st);
   launch_forces<Rr>(S, P, s->T, md ? 1 : 0, 0.5 * dt, st, !md);
   if (md && s->nvt) launch_nh_end(S, dt, st);
 }
@@ -516,27 +538,32 @@ static int capture_graph(ctbop_system* s, const PotParams<Rr>& P, bool md, doubl
   CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed));
   enqueue_front<Rr>(s, P, cs, md, dt);
   enqueue_middle<Rr>(s, P, cs);
-  cudaStreamCaptureStatus cst;
-  cudaGraph_t cg_graph;
-  const cudaGraphNode_t* deps = nullptr;
-  size_t ndeps = 0;
-  cudaError_t e = cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cg_graph, &deps, nullptr, &ndeps);
-  cudaGraphConditionalHandle handle;
-  if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&handle, cg_graph, 1, cudaGraphCondAssignDefault);
-  cudaGraphNodeParams cp = {cudaGraphNodeTypeConditional};
-  cp.conditional.handle = handle;
-  cp.conditional.type = cudaGraphCondTypeWhile;
-  cp.conditional.size = 1;
-  cudaGraphNode_t node;
-  if (e == cudaSuccess) e = cudaGraphAddNode(&node, cg_graph, deps, nullptr, ndeps, &cp);
-  if (e == cudaSuccess) e = cudaStreamUpdateCaptureDependencies(cs, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
-  if (e == cudaSuccess) {
-    cudaGraph_t body = cp.conditional.phGraph_out[0];
-    e = cudaStreamBeginCaptureToGraph(s->body_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
+  cudaError_t e = cudaSuccess;
+  if (s->S.solver != SOLVE_LAUNCHES) {
+    e = launch_cg_solve<Rr>(s->S, s->T, cg_tol(s), s->o.cg_max_iter, nullptr, cs);
+  } else {
+    cudaStreamCaptureStatus cst;
+    cudaGraph_t cg_graph;
+    const cudaGraphNode_t* deps = nullptr;
+    size_t ndeps = 0;
+    e = cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cg_graph, &deps, nullptr, &ndeps);
+    cudaGraphConditionalHandle handle;
+    if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&handle, cg_graph, 1, cudaGraphCondAssignDefault);
+    cudaGraphNodeParams cp = {cudaGraphNodeTypeConditional};
+    cp.conditional.handle = handle;
+    cp.conditional.type = cudaGraphCondTypeWhile;
+    cp.conditional.size = 1;
+    cudaGraphNode_t node;
+    if (e == cudaSuccess) e = cudaGraphAddNode(&node, cg_graph, deps, nullptr, ndeps, &cp);
+    if (e == cudaSuccess) e = cudaStreamUpdateCaptureDependencies(cs, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
     if (e == cudaSuccess) {
-      SolveCfg cfg{cg_tol(s), s->o.cg_max_iter, 1, handle};
-      launch_cg_iter<Rr>(s->S, cfg, s->body_stream);
-      e = cudaStreamEndCapture(s->body_stream, &body);
+      cudaGraph_t body = cp.conditional.phGraph_out[0];
+      e = cudaStreamBeginCaptureToGraph(s->body_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
+      if (e == cudaSuccess) {
+        SolveCfg cfg{cg_tol(s), s->o.cg_max_iter, 1, handle};
+        launch_cg_iter<Rr>(s->S, cfg, s->body_stream);
+        e = cudaStreamEndCapture(s->body_stream, &body);
+      }
     }
   }
   enqueue_back<Rr>(s, P, cs, md, dt, true);
@@ -561,12 +588,8 @@ static int run_direct(ctbop_system* s, const PotParams<Rr>& P, bool md, double d
   if (solve) {
     enqueue_middle<Rr>(s, P, st);
     SolveCfg cfg{cg_tol(s), s->o.cg_max_iter, 0, 0};
-    for (int it = 0; it < s->o.cg_max_iter + 4; it += 4) {
-      for (int k = 0; k < 4; ++k) launch_cg_iter<Rr>(s->S, cfg, st);
-      CK(cudaMemcpyAsync(s->h_int, s->S.cg_active, sizeof(int), cudaMemcpyDeviceToHost, st));
-      CK(cudaStreamSynchronize(st));
-      if (*s->h_int == 0) break;
-    }
+    int rc = solve_direct<Rr>(s, cfg, nullptr, st);
+    if (rc) return rc;
   } else {
     launch_bond<Rr>(s->S, P, st);
   }
@@ -789,18 +812,24 @@ static int profile_t(ctbop_system* s, const PotParams<Rr>& P, int64_t n, double 
     if (!rc) rc = timed(1, 12, [&] { launch_zero_acc(S, st); launch_rebuild<Rr>(S, P, st); });
     if (!rc) rc = timed(2, sizeof(Rr) == 4 ? 3 : 1, [&] { launch_bond<Rr>(S, P, st); });
     if (!rc) rc = timed(3, 1, [&] { launch_assemble<Rr>(S, P, s->T, st); });
-    if (!rc) rc = timed(4, S.precond ? 5 : 3, [&] {
+    const bool whole = S.solver != SOLVE_LAUNCHES;   // one kernel per solve, counted as the matrix passes
+    if (!rc) rc = timed(4, (S.precond ? 2 : 0) + (whole ? 0 : 3), [&] {
       if (S.precond) launch_block_setup<Rr>(S, st);
-      launch_cg_begin<Rr>(S, s->T, st, cg_tol(s));
+      if (!whole) launch_cg_begin<Rr>(S, s->T, st, cg_tol(s));
     });
-    for (int it = 0; it < s->o.cg_max_iter && !rc; ++it) {
+    if (!rc && whole) {
+      cudaError_t e = cudaSuccess;
+      rc = timed(5, 1, [&] { e = launch_cg_solve<Rr>(S, s->T, cfg.tol, cfg.max_iter, nullptr, st); });
+      CK(e);
+    }
+    for (int it = 0; !whole && it < s->o.cg_max_iter && !rc; ++it) {
       CK(cudaMemcpyAsync(s->h_int, S.cg_active, sizeof(int), cudaMemcpyDeviceToHost, st));
       CK(cudaStreamSynchronize(st));
       if (*s->h_int == 0) break;
       rc = timed(5, 1, [&] { launch_cg_mv<Rr>(S, st); });
       if (!rc) rc = timed(6, 1, [&] { launch_cg_up<Rr>(S, cfg, st); });
     }
-    if (!rc) rc = timed(7, 2, [&] { launch_cg_end<Rr>(S, st); });
+    if (!rc && !whole) rc = timed(7, 2, [&] { launch_cg_end<Rr>(S, st); });
     if (!rc) rc = timed(8, sizeof(Rr) == 4 ? 3 : 1, [&] { launch_cov_force<Rr>(S, P, s->T, st); });
     if (!rc) rc = timed(9, s->nvt ? 2 : 1, [&] {
       launch_coul_gather<Rr>(S, P, s->T, 1, 0.5 * dt, st, false);
@@ -1270,6 +1299,7 @@ int ctbop_step(ctbop_system* s, int64_t n_steps, double dt_fs) {
     }
     if (bits & CT_ERR_NONFINITE) { result = fail(s, CTBOP_ERR_NONFINITE, "non-finite energy, force or position"); done += n; break; }
     if (bits & CT_ERR_REV_MISSING) { result = fail(s, CTBOP_ERR_CUDA, "internal: asymmetric covalent list"); break; }
+    if (bits & CT_ERR_SOLVER) { result = fail(s, CTBOP_ERR_CUDA, "internal: the charge solve gave up waiting"); break; }
     done += n;
     s->steps += n;
     s->solves += n;
@@ -1416,6 +1446,7 @@ int ctbop_status(ctbop_system* s, ctbop_stats* st) {
     st->mean_mat = sc / S.N;
   }
   if (bits & CT_ERR_NONFINITE) return fail(s, CTBOP_ERR_NONFINITE, "non-finite energy, force or position");
+  if (bits & CT_ERR_SOLVER) return fail(s, CTBOP_ERR_CUDA, "internal: the charge solve gave up waiting");
   if (bits & CT_ERR_CG_MAXITER) return fail(s, CTBOP_ERR_CG_NOT_CONVERGED, "charge CG reached max_iter");
   return CTBOP_OK;
 }
@@ -1517,14 +1548,10 @@ static int param_grad_impl(ctbop_system* s, const double* w_E, const double* E_r
     double tol = cg_tol(s);
     if (fp32 && s->o.cg_tol <= 0) tol = std::max(tol, 2e-6 * vmax);
     SolveCfg cfg{tol, s->o.cg_max_iter, 0, 0};
-    launch_cg_begin<Rr>(S, s->T, st, cfg.tol, d_v);
-    for (int it = 0; it < s->o.cg_max_iter + 4; it += 4) {
-      for (int k = 0; k < 4; ++k) launch_cg_iter<Rr>(S, cfg, st);
-      CK(cudaMemcpyAsync(s->h_int, S.cg_active, sizeof(int), cudaMemcpyDeviceToHost, st));
-      CK(cudaStreamSynchronize(st));
-      if (*s->h_int == 0) break;
-    }
-    launch_cg_end<Rr>(S, st);
+    if (S.solver == SOLVE_LAUNCHES) launch_cg_begin<Rr>(S, s->T, st, cfg.tol, d_v);
+    rc = solve_direct<Rr>(s, cfg, d_v, st);
+    if (rc) return rc;
+    if (S.solver == SOLVE_LAUNCHES) launch_cg_end<Rr>(S, st);
     unsigned bits = 0;
     rc = read_err(s, bits);
     if (!rc && (bits & CT_ERR_CG_MAXITER)) rc = fail(s, CTBOP_ERR_CG_NOT_CONVERGED, "param_grad: adjoint CG reached max_iter");

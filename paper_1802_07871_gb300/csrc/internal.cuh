@@ -33,6 +33,7 @@
 #define CT_ERR_NONFINITE 8u
 #define CT_ERR_CG_MAXITER 16u
 #define CT_ERR_CODE_RANGE 32u
+#define CT_ERR_SOLVER 64u   // a barrier of the whole-solve kernel gave up
 
 namespace ct {
 

@@ -147,8 +147,19 @@ struct DevState {
   void* binv = nullptr;         // [ceil(N/32)][32][32] block inverses, row by row per block: FP16 (FP32 path) or FP64
   void* bsum = nullptr;         // Real[N]: row sums of the block inverses (d = M^-1 1)
   long long* precond_epoch = nullptr;   // rebuild count the block inverses were formed at (-1: never)
+  // charge solve: which form (plan_cg_solve), its blocks (per cluster or in
+  // all), groups of 32 atoms per block, atoms of the largest replica (cluster team)
+  int solver = 0, solve_blocks = 0, solve_per = 0, solve_maxn = 0;
+  int* solve_ctl = nullptr;     // [4], zero between solves (cgsolve.cu)
+  double* solve_part = nullptr; // [2][6][SOLVE_MAX_BLOCKS] partial sums of the grid-wide team
   void* stage = nullptr;        // [N * 24 bytes] staging for per-atom inputs and outputs in the caller's order
 };
+
+// The forms of the charge solve: two launches per iteration (cg.cu), or one
+// kernel per solve with a thread-block cluster per replica or all blocks on
+// one replica (cgsolve.cu).
+enum Solver { SOLVE_LAUNCHES = 0, SOLVE_CLUSTER = 1, SOLVE_GRID = 2 };
+#define SOLVE_MAX_BLOCKS 512
 
 struct SolveCfg {
   double tol;
@@ -165,6 +176,12 @@ template <class R> void launch_cg_begin(const DevState& S, const TypeParams& T, 
                                         const double* rhs = nullptr);
 template <class R> void launch_cg_iter(const DevState& S, const SolveCfg& cfg, cudaStream_t st);
 template <class R> void launch_cg_end(const DevState& S, cudaStream_t st);
+// The whole solve in one launch (S.solver not SOLVE_LAUNCHES); rhs as in launch_cg_begin.
+template <class R>
+cudaError_t launch_cg_solve(const DevState& S, const TypeParams& T, double tol, int max_iter, const double* rhs,
+                            cudaStream_t st);
+// Picks S.solver for the current layout (off: atom offsets, host) and list capacities.
+template <class R> cudaError_t plan_cg_solve(DevState& S, const int64_t* off);
 template <class R> void launch_cg_mv(const DevState& S, cudaStream_t st);
 template <class R> cudaError_t tune_cg_mv(DevState& S, cudaStream_t st, float* ms_out);
 template <class R> void launch_cg_up(const DevState& S, const SolveCfg& cfg, cudaStream_t st);
