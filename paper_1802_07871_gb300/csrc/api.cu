@@ -183,6 +183,7 @@ static void pack_params(const ctbop_params& p, double skin, PotParams<Rr>& P) {
     }
   P.rcoul = (Rr)p.r_coul;
   P.inv_rcoul = (Rr)(1.0 / p.r_coul);
+  P.rcoul2 = (Rr)(p.r_coul * p.r_coul);
   P.ke = (Rr)p.k_e;
   P.rall_list2 = (Rr)((p.r_coul + skin) * (p.r_coul + skin));
   P.rcore_list2 = p.r_coul > skin ? (Rr)((p.r_coul - skin) * (p.r_coul - skin)) : (Rr)0;

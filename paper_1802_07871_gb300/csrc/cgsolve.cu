@@ -170,16 +170,6 @@ __device__ inline unsigned long long shfl_xor_u64(unsigned long long v, int o) {
   return __shfl_xor_sync(CT_FULL, v, o);
 }
 
-// Two sums over a warp at once, a in lanes 0..15 and b in lanes 16..31: five
-// additions instead of ten.
-template <class R>
-__device__ inline R pair_sum(R a, R b) {
-  const bool up = (threadIdx.x & 16) != 0;
-  R v = (up ? b : a) + __shfl_xor_sync(CT_FULL, up ? a : b, 16);
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(CT_FULL, v, o);
-  return v;
-}
 // Two maxima likewise.
 __device__ inline float pair_max(float a, float b) {
   const bool up = (threadIdx.x & 16) != 0;

@@ -55,7 +55,7 @@ template <class R> struct PotParams {
   R gam[8][2], c2[8][2], d2[8][2], h[8][2], alpha[8][2], c2d2[8][2];
   // charge kernel
   R gshield3[4];                   // (gamma_i gamma_j)^(-3/2)
-  R rcoul, inv_rcoul, ke;
+  R rcoul, inv_rcoul, rcoul2, ke;
   R rall_list2;                    // (Rc + skin)^2
   R rcore_list2;                   // (Rc - skin)^2 (0 if Rc <= skin): entries inside stay inside Rc
                                    // until the next rebuild
@@ -106,12 +106,26 @@ template <> __device__ inline double ct_pow<double>(double x, double y) { return
 template <class R> __device__ inline R ct_sqrt(R x);
 template <> __device__ inline float ct_sqrt<float>(float x) { return sqrtf(x); }
 template <> __device__ inline double ct_sqrt<double>(double x) { return sqrt(x); }
-template <class R> __device__ inline R ct_cbrt(R x);
-template <> __device__ inline float ct_cbrt<float>(float x) { return cbrtf(x); }
-template <> __device__ inline double ct_cbrt<double>(double x) { return cbrt(x); }
 template <class R> __device__ inline R ct_rsqrt(R x);
 template <> __device__ inline float ct_rsqrt<float>(float x) { return rsqrtf(x); }
-template <> __device__ inline double ct_rsqrt<double>(double x) { return 1.0 / sqrt(x); }
+// FP64 reciprocal roots of the charge kernel, for positive x of moderate size
+// (r^2 and r^3 + gamma^-3: 0.1 to a few hundred). The FP64 pipe takes 64
+// cycles for a warp instruction on this GPU, so 1 / sqrt(x) and 1 / cbrt(x)
+// by root and division, with K and K' about 230 instructions per list entry,
+// made the charge-force pass 1.5 ms at 512 and at 19,555 atoms. Here a
+// hardware approximation y of x^(-1/n) (relative error near 2^-21) is refined
+// by one step of Householder's third-order iteration (A. S. Householder, The
+// Numerical Treatment of a Single Nonlinear Equation, 1970): with
+// e = 1 - x y^n, x^(-1/n) = y (1 - e)^(-1/n) = y (1 + e/n + (n+1) e^2 / (2 n^2)
+// + ...); the next term is below 1e-18. Five and six FP64 instructions, within
+// a few 1e-16 (checked against the library functions in the tests).
+__device__ inline double rsqrt_step(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y, e * fma(e, 0.375, 0.5), y);
+}
+template <> __device__ inline double ct_rsqrt<double>(double x) { return rsqrt_step(x); }
 template <class R> __device__ inline R ct_rcbrt(R x);
 // x^(-1/3) in FP32 for positive normal x (the charge kernel's
 // r^3 + gamma^-3, a few to a few hundred): a first guess 2^(-log2(x)/3) from
@@ -129,7 +143,16 @@ __device__ inline float rcbrt_newton(float x) {
   return fmaf(y * 0.333333343f, e, y);
 }
 template <> __device__ inline float ct_rcbrt<float>(float x) { return rcbrt_newton(x); }
-template <> __device__ inline double ct_rcbrt<double>(double x) { return 1.0 / cbrt(x); }
+__device__ inline double rcbrt_step(double x) {
+  float l = (float)x, f;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(l));
+  l *= -0.333333343f;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(l));
+  const double y = (double)f;
+  const double e = fma(-x, y * y * y, 1.0);
+  return fma(y, e * fma(e, 2.0 / 9.0, 1.0 / 3.0), y);
+}
+template <> __device__ inline double ct_rcbrt<double>(double x) { return rcbrt_step(x); }
 template <class R> __device__ inline R ct_cospi(R x);
 template <> __device__ inline float ct_cospi<float>(float x) { return cospif(x); }
 template <> __device__ inline double ct_cospi<double>(double x) { return cospi(x); }
@@ -154,46 +177,35 @@ __device__ inline void cutoff_fn(R r, R Rin, R Sout, R pi_SR, R& f, R& df) {
   df = -pi_SR * s * c;
 }
 
-// Shielded, tapered charge kernel K(r) and dK/dr.
-template <class R>
-__device__ inline void coul_fn(R r, R gs3, R inv_rc, R ke, R& K, R& dK) {
-  R x = r * inv_rc;
-  if (x >= R(1)) { K = R(0); dK = R(0); return; }
-  R x2 = x * x, x3 = x2 * x, x4 = x2 * x2;
-  R T = R(1) + x4 * (R(-35) + x * (R(84) + x * (R(-70) + R(20) * x)));
-  R xm = x - R(1);
-  R dT = R(140) * x3 * xm * xm * xm;
-  R r3 = r * r * r;
-  R D = ct_cbrt<R>(r3 + gs3);
-  R iD = R(1) / D;
-  K = ke * T * iD;
-  R iD3 = iD * iD * iD;
-  dK = ke * (dT * inv_rc * iD - T * r * r * iD3 * iD);
+// Shielded, tapered charge kernel K(r) = ke T(r/Rc) / (r^3 + gamma^-3)^(1/3).
+//
+// Past the charge cutoff? (r^2 against Rc^2; in FP64 the bits compared as
+// integers, the same order for positive values, off the FP64 pipe)
+__device__ inline bool past_cut(float r2, float rc2) { return !(r2 < rc2); }
+__device__ inline bool past_cut(double r2, double rc2) {
+  return __double_as_longlong(r2) >= __double_as_longlong(rc2);
 }
 
 // The same K(r) from r^2 for the streamed passes: 1/r and 1/(r^3 +
-// gamma^-3)^(1/3) come from the reciprocal root functions (FP32 path) instead
-// of a root and a division each. Returns r, 1/r, K and K'(r)/r.
+// gamma^-3)^(1/3) come from the reciprocal root functions. K = ke k and
+// K'/r = ke d with
+//   k = T iD, d = iD (140 x^2 (x - 1)^3 / Rc^2 - T r iD^3), x = r / Rc
+// (dT/dx = 140 x^3 (x - 1)^3, and x / r = 1 / Rc). Zero past the cutoff.
 template <class R>
-__device__ inline void coul_fn_r2(R r2, R gs3, R inv_rc, R ke, R& r, R& ir, R& K, R& dK_r) {
-  ir = ct_rsqrt<R>(r2);
-  r = r2 * ir;
-  R x = r * inv_rc;
-  if (x >= R(1)) { K = R(0); dK_r = R(0); return; }
-  R x2 = x * x, x3 = x2 * x, x4 = x2 * x2;
-  R T = R(1) + x4 * (R(-35) + x * (R(84) + x * (R(-70) + R(20) * x)));
-  R xm = x - R(1);
-  R dT = R(140) * x3 * xm * xm * xm;
-  R iD = ct_rcbrt<R>(r2 * r + gs3);
-  K = ke * T * iD;
-  R iD3 = iD * iD * iD;
-  dK_r = ke * (dT * inv_rc * iD * ir - T * r * iD3 * iD);
+__device__ inline void coul_kd_r2(R r2, R gs3, R inv_rc, R rc2, R& k, R& d) {
+  if (past_cut(r2, rc2)) { k = R(0); d = R(0); return; }
+  const R r = r2 * ct_rsqrt<R>(r2);
+  const R x = r * inv_rc, x2 = x * x, xm = x - R(1);
+  const R T = R(1) + (x2 * x2) * (R(-35) + x * (R(84) + x * (R(-70) + R(20) * x)));
+  const R iD = ct_rcbrt<R>(r2 * r + gs3);
+  k = T * iD;
+  d = iD * ((R(140) * inv_rc * inv_rc) * x2 * (xm * (xm * xm)) - (T * r) * (iD * (iD * iD)));
 }
 template <class R>
-__device__ inline R coul_K_r2(R r2, R gs3, R inv_rc, R ke) {
+__device__ inline R coul_K_r2(R r2, R gs3, R inv_rc, R rc2, R ke) {
+  if (past_cut(r2, rc2)) return R(0);
   R r = r2 * ct_rsqrt<R>(r2);
   R x = r * inv_rc;
-  if (x >= R(1)) return R(0);
   R x4 = (x * x) * (x * x);
   R T = R(1) + x4 * (R(-35) + x * (R(84) + x * (R(-70) + R(20) * x)));
   return ke * T * ct_rcbrt<R>(r2 * r + gs3);
@@ -320,6 +332,16 @@ __device__ inline double warp_sum(double v) {
 __device__ inline float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(CT_FULL, v, o);
+  return v;
+}
+// Two sums over a warp at once, a in lanes 0..15 and b in lanes 16..31: five
+// additions instead of ten.
+template <class R>
+__device__ inline R pair_sum(R a, R b) {
+  const bool up = (threadIdx.x & 16) != 0;
+  R v = (up ? b : a) + __shfl_xor_sync(CT_FULL, up ? a : b, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(CT_FULL, v, o);
   return v;
 }
 __device__ inline double warp_max(double v) {

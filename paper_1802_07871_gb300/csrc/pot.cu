@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(256)
     R r2 = rx * rx + ry * ry + rz * rz;
     int tj = (int)uj.w;
     int pb = ti * 2 + tj;
-    R m = coul_K_r2<R>(r2, P.gshield3[pb], P.inv_rcoul, P.ke);
+    R m = coul_K_r2<R>(r2, P.gshield3[pb], P.inv_rcoul, P.rcoul2, P.ke);
     R r = ct_sqrt<R>(r2);
     if (r < P.Sout[pb]) {
       R fc, dfc;
@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(256)
           R rx, ry, rz;
           rel_vec<R>(ui, uj[k], cc[k], hx, hy, hz, rx, ry, rz);
           R r2 = rx * rx + ry * ry + rz * rz;
-          R m = coul_K_r2<R>(r2, uj[k].w != R(0) ? gs_i1 : gs_i0, P.inv_rcoul, P.ke);
+          R m = coul_K_r2<R>(r2, uj[k].w != R(0) ? gs_i1 : gs_i0, P.inv_rcoul, P.rcoul2, P.ke);
           if (jc[k] == i) selfm += m;
           mat_store(M, (size_t)row * ld + i, jc[k], m);
         }
@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(256)
         R rx, ry, rz;
         rel_vec<R>(ui, uj[k], cc[k], hx, hy, hz, rx, ry, rz);
         R r2 = rx * rx + ry * ry + rz * rz;
-        R m = coul_K_r2<R>(r2, uj[k].w != R(0) ? gs_i1 : gs_i0, P.inv_rcoul, P.ke);
+        R m = coul_K_r2<R>(r2, uj[k].w != R(0) ? gs_i1 : gs_i0, P.inv_rcoul, P.rcoul2, P.ke);
         if (jc[k] == i) selfm += m;
         if (sizeof(R) == 8) {
           mat_store(M, (size_t)(e + k) * ld + i, jc[k], m);
@@ -495,6 +495,135 @@ __global__ void __launch_bounds__(256)
   R D = (R)(2.0 * by_type(T.J, ti)) + R(2) * wsum;
   Dg[i] = D;
   dinv[i] = R(1) / (D + selfm);
+}
+
+// The same matrix with G lanes per atom (8 or 32; 32 / G consecutive atoms
+// per warp, lane l * (32 / G) + a holding share l of atom a), for systems too
+// small to fill the chip with a thread per atom: a row's entries are dealt to
+// the lanes, a shell entry's place is its rank among the kept ones (ballots),
+// so the matrix has the same entries in the same places. FP64 is bound by its
+// pipe (64 cycles per warp instruction and scheduler): at 512 atoms a thread
+// per atom keeps 2 of 152 SMs busy (1,019 us; 21 with 32 lanes per atom).
+#define LG_T 256         // threads per block
+#define LG_B 4           // entries in flight per lane
+#define LG_FULL32 1000   // atoms per SM from which a thread per atom does (FP32)
+#define LG_FULL64 2000   // (FP64)
+template <class R, int G>
+__global__ void __launch_bounds__(LG_T)
+    k_assemble_g(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ u,
+                 const int* __restrict__ rep, const RepInfo* __restrict__ reps, const int2* __restrict__ nl,
+                 const int* __restrict__ ncov, const int* __restrict__ nfix, const int* __restrict__ nall,
+                 const int* __restrict__ rev, const typename Vec4<R>::T* __restrict__ bo, PotParams<R> P,
+                 TypeParams T, void* __restrict__ M, R* __restrict__ Dg, R* __restrict__ dinv,
+                 int* __restrict__ nmat) {
+  using R4 = typename Vec4<R>::T;
+  constexpr int AW = 32 / G;   // atoms per warp
+  const int lane = threadIdx.x & 31, a = lane % AW, l = lane / AW;
+  const int i = (int)((blockIdx.x * LG_T + threadIdx.x) >> 5) * AW + a;
+  const bool in = i < N;
+  unsigned mine = 0u;   // the lanes of this atom
+#pragma unroll
+  for (int k = 0; k < G; ++k) mine |= 1u << (k * AW);
+  mine <<= a;
+  const unsigned before = (1u << lane) - 1u;
+  R4 ui;
+  ui.x = ui.y = ui.z = ui.w = R(0);
+  R hx = R(0), hy = R(0), hz = R(0);
+  int nc = 0, nf = 0, na = 0;
+  if (in) {
+    ui = u[i];
+    const RepInfo& ri = reps[rep[i]];
+    hx = ri.hcf[0]; hy = ri.hcf[1]; hz = ri.hcf[2];
+    if (sizeof(R) == 8) { hx = (R)ri.hc[0]; hy = (R)ri.hc[1]; hz = (R)ri.hc[2]; }
+    nc = ncov[i];
+    nf = nfix[i];
+    na = nall[i];
+  }
+  const int ti = (int)ui.w;
+  const R gs_i0 = P.gshield3[ti * 2], gs_i1 = P.gshield3[ti * 2 + 1];
+  const int2* pl = nl + i;
+  R wsum = R(0), selfm = R(0);
+  // covalent entries: K minus twice the bond-order coupling w
+  for (int e = l; e < nc; e += G) {
+    const int2 jcd = __ldg(pl + (size_t)e * ld);
+    const int j = jcd.x;
+    const R4 uj = u[j];
+    R rx, ry, rz;
+    rel_vec<R>(ui, uj, jcd.y, hx, hy, hz, rx, ry, rz);
+    const R r2 = rx * rx + ry * ry + rz * rz;
+    const int pb = ti * 2 + (int)uj.w;
+    R m = coul_K_r2<R>(r2, P.gshield3[pb], P.inv_rcoul, P.rcoul2, P.ke);
+    const R r = ct_sqrt<R>(r2);
+    if (r < P.Sout[pb]) {
+      R fc, dfc;
+      cutoff_fn<R>(r, P.Rin[pb], P.Sout[pb], P.pi_SR[pb], fc, dfc);
+      const R fA = P.B[pb] * ct_exp<R>(-P.lam2[pb] * r);
+      const R bij = bo[(size_t)i * cap_cov + e].x;
+      const R bji = bo[(size_t)j * cap_cov + rev[(size_t)i * cap_cov + e]].x;
+      const R w = R(0.5) * P.kappa[pb] * fc * fA * (bij + bji);
+      m -= R(2) * w;
+      wsum += w;
+    }
+    if (j == i) selfm += m;
+    mat_store(M, (size_t)e * ld + i, j, m);
+  }
+  auto kernel = [&](const R4& uj, int cd) {
+    R rx, ry, rz;
+    rel_vec<R>(ui, uj, cd, hx, hy, hz, rx, ry, rz);
+    const R r2 = rx * rx + ry * ry + rz * rz;
+    return coul_K_r2<R>(r2, uj.w != R(0) ? gs_i1 : gs_i0, P.inv_rcoul, P.rcoul2, P.ke);
+  };
+  // core entries, and in FP64 the shell too: stored at their list row
+  const int n1 = sizeof(R) == 8 ? na : nf;
+  for (int e0 = nc + l; e0 < n1; e0 += G * LG_B) {
+    int2 jc[LG_B];
+    R4 uj[LG_B];
+#pragma unroll
+    for (int k = 0; k < LG_B; ++k)
+      jc[k] = e0 + k * G < n1 ? __ldg(pl + (size_t)(e0 + k * G) * ld) : make_int2(i, pack_code(0, 0, 0));
+#pragma unroll
+    for (int k = 0; k < LG_B; ++k) uj[k] = u[jc[k].x];
+#pragma unroll
+    for (int k = 0; k < LG_B; ++k) {
+      const int e = e0 + k * G;
+      if (e < n1) {
+        const R m = kernel(uj[k], jc[k].y);
+        if (jc[k].x == i) selfm += m;
+        mat_store(M, (size_t)e * ld + i, jc[k].x, m);
+      }
+    }
+  }
+  if (sizeof(R) == 4) {   // shell entries inside the cutoff, packed after the core
+    int em = nf;
+    const int rounds = (int)__reduce_max_sync(CT_FULL, (unsigned)((na - nf + G - 1) / G));
+    for (int q = 0; q < rounds; ++q) {
+      const int e = nf + q * G + l;
+      R m = R(0);
+      int j = i;
+      if (e < na) {
+        const int2 jc = __ldg(pl + (size_t)e * ld);
+        j = jc.x;
+        m = kernel(u[j], jc.y);
+      }
+      const unsigned kept = __ballot_sync(CT_FULL, m != R(0)) & mine;
+      if (m != R(0)) {
+        if (j == i) selfm += m;
+        mat_store(M, (size_t)(em + __popc(kept & before)) * ld + i, j, m);
+      }
+      em += __popc(kept);
+    }
+    if (in && l == 0) nmat[i] = em;
+  }
+#pragma unroll
+  for (int o = AW; o < 32; o <<= 1) {
+    wsum += __shfl_xor_sync(CT_FULL, wsum, o);
+    selfm += __shfl_xor_sync(CT_FULL, selfm, o);
+  }
+  if (in && l == 0) {
+    const R D = (R)(2.0 * by_type(T.J, ti)) + R(2) * wsum;
+    Dg[i] = D;
+    dinv[i] = R(1) / (D + selfm);
+  }
 }
 
 // ---------------------------------------------------------------- covalent forces
@@ -749,7 +878,7 @@ __global__ void __launch_bounds__(256, gather_min_blocks<PB, VIR>())
     R hx = ri.hcf[0], hy = ri.hcf[1], hz = ri.hcf[2];
     if (sizeof(R) == 8) { hx = (R)ri.hc[0]; hy = (R)ri.hc[1]; hz = (R)ri.hc[2]; }
     int nc = ncov[i], na = nall[i];
-    R qi = qr[i];
+    R qi = P.ke * qr[i];
     R fx = R(0), fy = R(0), fz = R(0);
     CompSum<R> ec;
     R w[9];
@@ -766,8 +895,8 @@ __global__ void __launch_bounds__(256, gather_min_blocks<PB, VIR>())
       R rx, ry, rz;
       rel_vec<R>(ui, uj, jcd.y, hx, hy, hz, rx, ry, rz);
       R r2 = rx * rx + ry * ry + rz * rz;
-      R r, ir, K, c;
-      coul_fn_r2<R>(r2, uj.w != R(0) ? gs_i1 : gs_i0, P.inv_rcoul, P.ke, r, ir, K, c);
+      R K, c;
+      coul_kd_r2<R>(r2, uj.w != R(0) ? gs_i1 : gs_i0, P.inv_rcoul, P.rcoul2, K, c);
       R qq = qi * qr[j];
       c *= qq;
       R4 go = gslot[(size_t)i * cap_cov + e];
@@ -818,8 +947,8 @@ __global__ void __launch_bounds__(256, gather_min_blocks<PB, VIR>())
           R rx, ry, rz;
           rel_vec<R>(ui, uj[k], cc[k], hx, hy, hz, rx, ry, rz);
           R r2 = rx * rx + ry * ry + rz * rz;
-          R r, ir, K, c;
-          coul_fn_r2<R>(r2, uj[k].w != R(0) ? gs_i1 : gs_i0, P.inv_rcoul, P.ke, r, ir, K, c);
+          R K, c;
+          coul_kd_r2<R>(r2, uj[k].w != R(0) ? gs_i1 : gs_i0, P.inv_rcoul, P.rcoul2, K, c);
           R qq = qi * qj[k];
           c *= qq;
           fx += c * rx; fy += c * ry; fz += c * rz;
@@ -864,6 +993,187 @@ __global__ void __launch_bounds__(256, gather_min_blocks<PB, VIR>())
   }
   fold();
   lane_flush<RA_STRIDE>(acc, rep_acc, RA_STRIDE);
+}
+
+// The same with G lanes per atom (lanes as in k_assemble_g): a row's entries
+// are dealt to the lanes, their sums joined by shuffles (the energies with
+// their compensation), and one warp of the block then takes the block's atoms
+// through the FP64 epilogue with full lanes.
+template <class R, int G, bool VIR>
+__global__ void __launch_bounds__(LG_T)
+    k_coul_gather_g(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ u,
+                    const int* __restrict__ rep, const RepInfo* __restrict__ reps, const int2* __restrict__ nl,
+                    const int* __restrict__ ncov, const int* __restrict__ nall,
+                    const int* __restrict__ rev, const typename Vec4<R>::T* __restrict__ gslot,
+                    const R* __restrict__ qr, PotParams<R> P, TypeParams T, int kick, double half_dt,
+                    const uint8_t* __restrict__ frozen, double* __restrict__ F, double* __restrict__ v,
+                    double* __restrict__ e_atom, double* __restrict__ rep_acc, unsigned* __restrict__ err,
+                    const double* __restrict__ nh) {
+  using R4 = typename Vec4<R>::T;
+  constexpr int AW = 32 / G, AB = LG_T / 32 * AW;   // atoms per warp, per block
+  constexpr int NS = VIR ? 14 : 5;
+  __shared__ R s_v[NS][AB];   // force, energy (sum, compensation), virial
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, a = lane % AW, l = lane / AW;
+  const int i = ((int)blockIdx.x * (LG_T / 32) + warp) * AW + a;
+  R s[NS];
+#pragma unroll
+  for (int k = 0; k < NS; ++k) s[k] = R(0);
+  CompSum<R> ec;
+  if (i < N) {
+    const R4 ui = u[i];
+    const int ti = (int)ui.w;
+    const RepInfo& ri = reps[rep[i]];
+    R hx = ri.hcf[0], hy = ri.hcf[1], hz = ri.hcf[2];
+    if (sizeof(R) == 8) { hx = (R)ri.hc[0]; hy = (R)ri.hc[1]; hz = (R)ri.hc[2]; }
+    const int nc = ncov[i], na = nall[i];
+    const int2* pl = nl + i;
+    const R gs_i0 = P.gshield3[ti * 2], gs_i1 = P.gshield3[ti * 2 + 1];
+    // charges: qj K and qj K'/r are summed, (ke / 2) qi and ke qi applied once per lane
+    auto add = [&](R rx, R ry, R rz, R wj, R qj, R& en) {
+      const R r2 = rx * rx + ry * ry + rz * rz;
+      R K, c;
+      coul_kd_r2<R>(r2, wj != R(0) ? gs_i1 : gs_i0, P.inv_rcoul, P.rcoul2, K, c);
+      c *= qj;
+      // (explicit: the variants with and without the virial round alike)
+      s[0] = fma(c, rx, s[0]); s[1] = fma(c, ry, s[1]); s[2] = fma(c, rz, s[2]);
+      en = qj * K;
+      if (VIR) {
+        const R tx = c * rx, ty = c * ry, tz = c * rz;
+        s[5] += rx * tx; s[6] += rx * ty; s[7] += rx * tz;
+        s[8] += ry * tx; s[9] += ry * ty; s[10] += ry * tz;
+        s[11] += rz * tx; s[12] += rz * ty; s[13] += rz * tz;
+      }
+    };
+    for (int e0 = l; e0 < na; e0 += G * LG_B) {
+      int2 jc[LG_B];
+      R4 uj[LG_B];
+      R qj[LG_B], en[LG_B];
+#pragma unroll
+      for (int k = 0; k < LG_B; ++k)
+        jc[k] = e0 + k * G < na ? __ldg(pl + (size_t)(e0 + k * G) * ld) : make_int2(i, pack_code(0, 0, 0));
+#pragma unroll
+      for (int k = 0; k < LG_B; ++k) {
+        uj[k] = u[jc[k].x];
+        qj[k] = qr[jc[k].x];
+      }
+#pragma unroll
+      for (int k = 0; k < LG_B; ++k) {
+        en[k] = R(0);
+        if (e0 + k * G < na) {
+          R rx, ry, rz;
+          rel_vec<R>(ui, uj[k], jc[k].y, hx, hy, hz, rx, ry, rz);
+          add(rx, ry, rz, uj[k].w, qj[k], en[k]);
+        }
+      }
+      if (sizeof(R) == 4) {
+#pragma unroll
+        for (int k = 0; k < LG_B; ++k) ec.add(en[k]);
+      } else {   // (FP64: the batch first, then one compensated addition)
+        ec.add((en[0] + en[1]) + (en[2] + en[3]));
+      }
+    }
+    const R qi = P.ke * qr[i], hq = R(0.5) * qi;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) s[k] *= qi;
+    if (VIR) {
+#pragma unroll
+      for (int k = 5; k < 14; ++k) s[k] *= -hq;
+    }
+    s[3] = hq * ec.s;
+    s[4] = hq * ec.c;
+    // bonds: own slot less the partner's slot that points back
+    for (int e = l; e < nc; e += G) {
+      const int2 jc = __ldg(pl + (size_t)e * ld);
+      const R4 go = gslot[(size_t)i * cap_cov + e];
+      const R4 gr = gslot[(size_t)jc.x * cap_cov + rev[(size_t)i * cap_cov + e]];
+      s[0] += go.x - gr.x; s[1] += go.y - gr.y; s[2] += go.z - gr.z;
+      if (VIR) {
+        R rx, ry, rz;
+        rel_vec<R>(ui, u[jc.x], jc.y, hx, hy, hz, rx, ry, rz);
+        s[5] -= rx * go.x; s[6] -= rx * go.y; s[7] -= rx * go.z;
+        s[8] -= ry * go.x; s[9] -= ry * go.y; s[10] -= ry * go.z;
+        s[11] -= rz * go.x; s[12] -= rz * go.y; s[13] -= rz * go.z;
+      }
+    }
+  }
+#pragma unroll
+  for (int o = AW; o < 32; o <<= 1) {
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+      if (k == 3 || k == 4) continue;
+      s[k] += __shfl_xor_sync(CT_FULL, s[k], o);
+    }
+    // the energies' sums with the rounding error of their addition (TwoSum)
+    const R b = __shfl_xor_sync(CT_FULL, s[3], o), cb = __shfl_xor_sync(CT_FULL, s[4], o);
+    const R t = s[3] + b, bb = t - s[3];
+    s[4] = (s[4] + cb) + ((s[3] - (t - bb)) + (b - bb));
+    s[3] = t;
+  }
+  if (l == 0) {
+#pragma unroll
+    for (int k = 0; k < NS; ++k) s_v[k][warp * AW + a] = s[k];
+  }
+  __syncthreads();
+  if (warp != 0) return;
+  const int ie = (int)blockIdx.x * AB + lane;
+  const bool in = lane < AB && ie < N;
+  int rid = -1;
+  double ea = 0.0, ke = 0.0;
+  R f2 = R(0);
+  if (in) {
+    rid = rep[ie];
+    const int ti = (int)u[ie].w;
+    const R fx = s_v[0][lane], fy = s_v[1][lane], fz = s_v[2][lane];
+    const double Fx = fx, Fy = fy, Fz = fz;
+    F[3 * ie] = Fx; F[3 * ie + 1] = Fy; F[3 * ie + 2] = Fz;
+    ea = e_atom[ie] + ((double)s_v[3][lane] + (double)s_v[4][lane]);
+    e_atom[ie] = ea;
+    const bool bad_e = (__double_as_longlong(ea) & 0x7ff0000000000000ll) == 0x7ff0000000000000ll;
+    if (bad_e || !isfinite(fx) || !isfinite(fy) || !isfinite(fz)) atomicOr(err, CT_ERR_NONFINITE);
+    f2 = fx * fx + fy * fy + fz * fz;
+    double vx = v[3 * ie], vy = v[3 * ie + 1], vz = v[3 * ie + 2];
+    if (kick && !frozen[ie]) {
+      const double sc = half_dt * by_type(T.inv_mass_acc, ti);
+      vx += sc * Fx; vy += sc * Fy; vz += sc * Fz;
+      const double* h = nh + (size_t)rid * NH_STRIDE;
+      if (h[NH_ON] != 0.0) {   // NVT: the second velocity scaling, exp(-xi' dt/2)
+        const double sv = exp(-half_dt * h[NH_XIH]);
+        vx *= sv; vy *= sv; vz *= sv;
+      }
+      v[3 * ie] = vx; v[3 * ie + 1] = vy; v[3 * ie + 2] = vz;
+    }
+    ke = 0.5 * by_type(T.mass, ti) * (vx * vx + vy * vy + vz * vz);   // of the current velocities
+  }
+  const int r0 = __shfl_sync(CT_FULL, rid, 0);
+  if (__all_sync(CT_FULL, rid == r0 || !in)) {
+    double* out = rep_acc + (size_t)max(r0, 0) * RA_STRIDE;
+    const double ek = pair_sum(ea, ke);   // lanes 0..15 the energy, 16..31 the kinetic energy
+    f2 = warp_sum(f2);
+    if (r0 >= 0) {
+      if (lane == 0) {
+        atomicAdd(out + RA_E, ek);
+        atomicAdd(out + RA_F2, (double)f2);
+      } else if (lane == 16) {
+        atomicAdd(out + RA_KE, ek);
+      }
+    }
+    if (VIR) {
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {
+        const R w = warp_sum(in ? s_v[NS - 9 + k][lane] : R(0));
+        if (lane == 0 && r0 >= 0) atomicAdd(out + RA_W + k, (double)w);
+      }
+    }
+  } else if (in) {   // a replica boundary inside the block
+    double* out = rep_acc + (size_t)rid * RA_STRIDE;
+    atomicAdd(out + RA_E, ea);
+    atomicAdd(out + RA_KE, ke);
+    atomicAdd(out + RA_F2, (double)f2);
+    if (VIR) {
+#pragma unroll
+      for (int k = 0; k < 9; ++k) atomicAdd(out + RA_W + k, (double)s_v[NS - 9 + k][lane]);
+    }
+  }
 }
 
 // FP64 offsets of every atom from its cell's origin (the layout of u), for
@@ -946,14 +1256,25 @@ void launch_bond(const DevState& S, const PotParams<R>& P, cudaStream_t st) {
   else launch_bond_g<R, 8>(S, P, st);
 }
 
+// Lanes per atom in the assembly and the charge-force gather: 1 (a thread
+// per atom, entries in flight per thread tuned) where that fills the chip,
+// else 8 or 32.
+template <class R>
+static int row_lanes(const DevState& S) {
+  const int full = S.nsm * (sizeof(R) == 4 ? LG_FULL32 : LG_FULL64);
+  return S.N <= S.nsm * 32 ? 32 : S.N <= full ? 8 : 1;
+}
+
 template <class R>
 void launch_assemble(const DevState& S, const PotParams<R>& P, const TypeParams& T, cudaStream_t st) {
   if (S.N == 0) return;
 #define ASM_ARGS                                                                                        \
   S.N, S.cap_cov, S.ld, (const typename Vec4<R>::T*)S.u, S.rep, S.reps, S.nl, S.ncov, S.nfix, S.nall, S.rev, \
       (const typename Vec4<R>::T*)S.bo, P, T, S.M, (R*)S.Dg, (R*)S.dinv, S.nmat
-  const int g = (S.N + 255) / 256;
-  if (S.asm_batch == 4) k_assemble<R, 4><<<g, 256, 0, st>>>(ASM_ARGS);
+  const int g = (S.N + 255) / 256, lanes = row_lanes<R>(S), per = LG_T / lanes;
+  if (lanes == 32) k_assemble_g<R, 32><<<(S.N + per - 1) / per, LG_T, 0, st>>>(ASM_ARGS);
+  else if (lanes == 8) k_assemble_g<R, 8><<<(S.N + per - 1) / per, LG_T, 0, st>>>(ASM_ARGS);
+  else if (S.asm_batch == 4) k_assemble<R, 4><<<g, 256, 0, st>>>(ASM_ARGS);
   else if (S.asm_batch == 16) k_assemble<R, 16><<<g, 256, 0, st>>>(ASM_ARGS);
   else k_assemble<R, 8><<<g, 256, 0, st>>>(ASM_ARGS);
 #undef ASM_ARGS
@@ -994,17 +1315,26 @@ template <class R>
 void launch_coul_gather(const DevState& S, const PotParams<R>& P, const TypeParams& T, int kick, double half_dt,
                         cudaStream_t st, bool virial) {
   if (S.N == 0) return;
+  const int lanes = row_lanes<R>(S);
   auto go = [&](auto kernel) {
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 256, 0) != cudaSuccess || occ < 1) occ = 1;
-    long long tiles = ((long long)S.N + 255) / 256, slots = (long long)S.nsm * occ;
-    int grid = (int)(tiles < slots ? tiles : slots);
+    int occ = 0, grid = 0;
+    if (lanes > 1) {
+      grid = (S.N + LG_T / lanes - 1) / (LG_T / lanes);
+    } else {
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 256, 0) != cudaSuccess || occ < 1) occ = 1;
+      long long tiles = ((long long)S.N + 255) / 256, slots = (long long)S.nsm * occ;
+      grid = (int)(tiles < slots ? tiles : slots);
+    }
     kernel<<<grid, 256, 0, st>>>(
         S.N, S.cap_cov, S.ld, (const typename Vec4<R>::T*)S.u, S.rep, S.reps, S.nl,
         S.ncov, S.nall, S.rev, (const typename Vec4<R>::T*)S.gslot, (const R*)S.qr, P, T, kick, half_dt,
         S.frozen, S.F, S.v, S.e_atom, S.rep_acc, S.err, S.nh);
   };
-  if (virial) {
+  if (lanes == 32) {
+    if (virial) go(k_coul_gather_g<R, 32, true>); else go(k_coul_gather_g<R, 32, false>);
+  } else if (lanes == 8) {
+    if (virial) go(k_coul_gather_g<R, 8, true>); else go(k_coul_gather_g<R, 8, false>);
+  } else if (virial) {
     if (S.gather_batch == 4) go(k_coul_gather<R, 4, true>);
     else if (S.gather_batch == 6) go(k_coul_gather<R, 6, true>);
     else go(k_coul_gather<R, 8, true>);
