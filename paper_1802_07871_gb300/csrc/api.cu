@@ -1859,13 +1859,25 @@ int ctbop_rings(ctbop_system* s, double bond_cut, int32_t max_size, int64_t cap,
   unsigned long long* d_cnt = nullptr;
   Scratch scr(s->stream, s->pool);
   CK(scr.alloc(&d_out, (size_t)std::max<int64_t>(cap, 1)));
-  CK(scr.alloc(&d_cnt, 1));
-  CK(zero_async(s, d_cnt, sizeof(unsigned long long)));
-  if (s->mixed) launch_rings<float>(s->S, bond_cut, max_size, d_out, cap, d_cnt, s->stream);
-  else launch_rings<double>(s->S, bond_cut, max_size, d_out, cap, d_cnt, s->stream);
-  CK(cudaGetLastError());
-  unsigned long long n = 0;
-  CK(sync_copy(s, &n, d_cnt, sizeof(n), cudaMemcpyDeviceToHost));
+  CK(scr.alloc(&d_cnt, 2));
+  CK(zero_async(s, d_cnt, 2 * sizeof(unsigned long long)));
+  CK(s->mixed ? launch_rings<float>(s->S, bond_cut, max_size, d_out, cap, d_cnt, s->stream)
+              : launch_rings<double>(s->S, bond_cut, max_size, d_out, cap, d_cnt, s->stream));
+  unsigned long long got[2] = {0, 0};
+  CK(sync_copy(s, got, d_cnt, sizeof(got), cudaMemcpyDeviceToHost));
+  // atoms with more surroundings than a table in shared memory holds
+  int slots = RING_WIDE_SLOTS;
+  for (int pass = 0; got[1] > 0; ++pass, slots *= 8) {
+    if (pass > 4) return fail(s, CTBOP_ERR_OOM, "rings: the bond network is too dense");
+    unsigned char* tables = nullptr;
+    Scratch wide(s->stream, s->pool);
+    CK(wide.alloc(&tables, rings_wide_bytes(s->S, s->mixed, slots)));
+    CK(zero_async(s, d_cnt + 1, sizeof(unsigned long long)));
+    CK(s->mixed ? launch_rings_wide<float>(s->S, pass, (int)got[1], slots, tables, max_size, d_out, cap, d_cnt, s->stream)
+                : launch_rings_wide<double>(s->S, pass, (int)got[1], slots, tables, max_size, d_out, cap, d_cnt, s->stream));
+    CK(sync_copy(s, got, d_cnt, sizeof(got), cudaMemcpyDeviceToHost));
+  }
+  const unsigned long long n = got[0];
   int64_t m = std::min<int64_t>((int64_t)n, cap);
   if (m > 0) CK(sync_copy(s, out, d_out, sizeof(ctbop_ring) * m, cudaMemcpyDeviceToHost));
   *n_rings = (int64_t)n;

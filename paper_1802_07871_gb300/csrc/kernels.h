@@ -241,11 +241,19 @@ void launch_fire_reduce(const DevState& S, double* fire, const FireCfg& cfg, int
 template <class R>
 void launch_fire_move(const DevState& S, const TypeParams& T, const double* fire, double half_skin2,
                       cudaStream_t st);
-// Primitive C rings (csrc/rings.cu): records appended through *count (the
-// total, which may exceed cap; records past cap are dropped).
+// Primitive C rings (csrc/rings.cu): records appended through count[0] (the
+// total, which may exceed cap; records past cap are dropped). count[1] atoms
+// are left over: launch_rings_wide searches them (pass 0, 1, ...) with tables
+// of `slots` places (a power of two) in rings_wide_bytes of device memory, and
+// leaves in count[1], cleared before, those that want larger ones.
 template <class R>
-void launch_rings(const DevState& S, double bond_cut, int max_size, ::ctbop_ring* out, long long cap,
-                  unsigned long long* count, cudaStream_t st);
+cudaError_t launch_rings(const DevState& S, double bond_cut, int max_size, ::ctbop_ring* out, long long cap,
+                         unsigned long long* count, cudaStream_t st);
+#define RING_WIDE_SLOTS 4096
+size_t rings_wide_bytes(const DevState& S, bool fp32, int slots);
+template <class R>
+cudaError_t launch_rings_wide(const DevState& S, int pass, int n_queue, int slots, void* tables, int max_size,
+                              ::ctbop_ring* out, long long cap, unsigned long long* count, cudaStream_t st);
 // Storage order (csrc/order.cu): dst[k] = src[order[k]] (to_storage) or
 // dst[order[k]] = src[k], elements of 1, 4, 8 or 24 bytes.
 cudaError_t launch_permute(int N, const int* order, const void* src, void* dst, int elem_bytes, bool to_storage,

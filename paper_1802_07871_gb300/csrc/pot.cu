@@ -506,8 +506,9 @@ __global__ void __launch_bounds__(256)
 // per atom keeps 2 of 152 SMs busy (1,019 us; 21 with 32 lanes per atom).
 #define LG_T 256         // threads per block
 #define LG_B 4           // entries in flight per lane
-#define LG_FULL32 1000   // atoms per SM from which a thread per atom does (FP32)
-#define LG_FULL64 2000   // (FP64)
+#define LG_FULL32 1300   // atoms per SM up to which FP32 takes 8 lanes per atom (at 158,391 atoms 172 + 161 us
+                         // against 190 + 205; at 1,005,466 atoms 2,410 + 1,183 against 938 + 970)
+#define LG_FULL64 2000   // the same for FP64 (its rows are bound by the FP64 pipe, not by their loads)
 template <class R, int G>
 __global__ void __launch_bounds__(LG_T)
     k_assemble_g(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ u,
