@@ -644,7 +644,7 @@ __global__ void __launch_bounds__(256)
 }
 
 // Element-wise update; the sums and maxima for the next c and the test.
-// Threads take 256-atom tiles strided over the grid; per-thread partial sums
+// Blocks take consecutive 256-atom tiles (tile_range); per-thread partial sums
 // in the working precision (a few atoms each), FP64 across warps and blocks.
 // The iterate's change dq = q - q0 is accumulated in the working precision
 // (it is small next to q) and added to the FP64 q once, after the loop, so
@@ -682,7 +682,9 @@ __global__ void __launch_bounds__(256)
   int crid = -1;
   R a = R(0), b = R(0), c = R(0), mprev = R(0);
   R part[3] = {R(0), R(0), R(0)};   // sum y, sum r, sum r^2
-  for (int t = blockIdx.x; (long long)t * 256 < N; t += gridDim.x) {
+  int t0, t1;
+  tile_range(N, t0, t1);
+  for (int t = t0; t < t1; ++t) {
     int i = t * 256 + (int)threadIdx.x;
     int rid = i < N ? rep[i] : -1;
     bool act = rid >= 0 && !conv[rid];
@@ -753,7 +755,9 @@ __global__ void __launch_bounds__(256) k_cg_qsum(int N, const int* __restrict__ 
                                                  const R* __restrict__ dqv, double* __restrict__ cg) {
   RepAcc<1> acc;
   acc.init();
-  for (int t = blockIdx.x; (long long)t * 256 < N; t += gridDim.x) {
+  int t0, t1;
+  tile_range(N, t0, t1);
+  for (int t = t0; t < t1; ++t) {
     int i = t * 256 + (int)threadIdx.x;
     if (i >= N) break;
     acc.to(rep[i], cg + CG_SQF, CG_STRIDE);

@@ -145,17 +145,6 @@ template <> struct PartSum<double> {
   __device__ inline double lo() const { return 0.0; }
 };
 
-// 1 / x for a finite non-zero x: the hardware's approximate reciprocal and two
-// Newton-Raphson steps (four FP64 instructions; the FP64 pipe takes 64 cycles
-// for each on this GPU, and a division is twice as many on the critical path
-// of every iteration).
-__device__ inline double recip(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  y = fma(y, fma(-x, y, 1.0), y);
-  return fma(y, fma(-x, y, 1.0), y);
-}
-
 // Order-preserving map of doubles to unsigned integers: maxima are taken on
 // integers (an FP64 maximum costs 97 cycles here).
 __device__ inline unsigned long long key_of(double x) {

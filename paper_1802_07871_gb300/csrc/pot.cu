@@ -170,7 +170,7 @@ k_bond(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ u,
   __shared__ int s_nstiff, s_base, s_nflag, s_fbase;
   if (threadIdx.x == 0) { s_nstiff = 0; s_nflag = 0; }
   int g = threadIdx.x / G, l = threadIdx.x % G;
-  // layout: R4 (ux,uy,uz,r)[APB_][cap] | R fc | int type | int live list
+  // layout: R4 (direction, r)[APB_][cap] | R fc | int type | int live list
   R4* s_u = reinterpret_cast<R4*>(smem_raw);
   R* s_fc = reinterpret_cast<R*>(s_u + (size_t)APB_ * cap_cov);
   int* s_t = reinterpret_cast<int*>(s_fc + (size_t)APB_ * cap_cov);
@@ -212,8 +212,9 @@ k_bond(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ u,
                     (float)P.pi_SR[pb], f, df);
         fc = (R)f;
       }
-      R4 w;
-      w.x = rx; w.y = ry; w.z = rz; w.w = r;
+      const R ir = inv(r);
+      R4 w;   // the bond's direction and length
+      w.x = rx * ir; w.y = ry * ir; w.z = rz * ir; w.w = r;
       s_u[e] = w;
       s_fc[e] = fc;
       s_t[e] = tj;
@@ -244,7 +245,7 @@ k_bond(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ u,
       }
       if (acc && (compressed || ue.w > P.Rin[pb])) my_flag = 1;
     }
-    R re = ue.w, ire = R(1) / re;
+    R re = ue.w;
     R z1 = R(0), z2 = R(0);
     int tbase = pb * 2;
     for (int kk = 0; kk < nlive; ++kk) {
@@ -253,18 +254,18 @@ k_bond(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ u,
       R fck = s_fc[k];
       R4 uk = s_u[k];
       int tri = tbase + s_t[k];
-      R ct = (ue.x * uk.x + ue.y * uk.y + ue.z * uk.z) * ire / uk.w;
+      R ct = ue.x * uk.x + ue.y * uk.y + ue.z * uk.z;
       R dr = re - uk.w;
       {
         R hm = P.h[tri][0] - ct;
         R hm2 = hm * hm;
-        R ang = P.gam[tri][0] * (R(1) + P.c2d2[tri][0] * hm2 / (P.d2[tri][0] + hm2));
+        R ang = P.gam[tri][0] * (R(1) + P.c2d2[tri][0] * hm2 * inv(P.d2[tri][0] + hm2));
         z1 += fck * ang * ct_exp<R>(P.alpha[tri][0] * dr);
       }
       {
         R hm = P.h[tri][1] - ct;
         R hm2 = hm * hm;
-        R ang = P.gam[tri][1] * (R(1) + P.c2d2[tri][1] * hm2 / (P.d2[tri][1] + hm2));
+        R ang = P.gam[tri][1] * (R(1) + P.c2d2[tri][1] * hm2 * inv(P.d2[tri][1] + hm2));
         z2 += fck * ang * ct_exp<R>(P.alpha[tri][1] * dr);
       }
     }
@@ -645,7 +646,7 @@ k_cov_force(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ 
   constexpr int APB_ = CB / G;
   extern __shared__ __align__(32) unsigned char smem_raw[];
   int g = threadIdx.x / G, l = threadIdx.x % G;
-  // layout: R4 u[APB_][cap] | R2 D[APB_][cap] | R fc | R dfc | R pair dE/dr | int type | int live list
+  // layout: R4 (direction, r)[APB_][cap] | R2 D[APB_][cap] | R fc | R dfc | R pair dE/dr | int type | int live list
   R4* s_u = reinterpret_cast<R4*>(smem_raw);
   R2* s_D = reinterpret_cast<R2*>(s_u + (size_t)APB_ * cap_cov);
   R* s_fc = reinterpret_cast<R*>(s_D + (size_t)APB_ * cap_cov);
@@ -718,8 +719,9 @@ k_cov_force(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ 
         D.x = pre * bb.y;
         D.y = pre * bb.z;
       }
-      R4 w;
-      w.x = rx; w.y = ry; w.z = rz; w.w = r;
+      const R ir = inv(r);
+      R4 w;   // the bond's direction and length
+      w.x = rx * ir; w.y = ry * ir; w.z = rz * ir; w.w = r;
       s_u[e] = w;
       s_D[e] = D;
       s_fc[e] = fc;
@@ -744,8 +746,8 @@ k_cov_force(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ 
       typename Vec4<O>::T out;
       out.x = O(0); out.y = O(0); out.z = O(0); out.w = O(0);
       {
-        R irx = R(1) / rx;
-        R hx_ = ux.x * irx, hy_ = ux.y * irx, hz_ = ux.z * irx;
+        const R irx = inv(rx);
+        const R hx_ = ux.x, hy_ = ux.y, hz_ = ux.z;
         R2 Dx = s_D[e];
         R dfcx = s_dfc[e];
         int tx = s_t[e];
@@ -756,43 +758,38 @@ k_cov_force(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ 
           if (k == e) continue;
           R fck = s_fc[k];
           R4 uk = s_u[k];
-          R rk = uk.w, irk = R(1) / rk;
-          R kx = uk.x * irk, ky = uk.y * irk, kz = uk.z * irk;
+          const R rk = uk.w, kx = uk.x, ky = uk.y, kz = uk.z;
           R ct = hx_ * kx + hy_ * ky + hz_ * kz;
           int tk = s_t[k];
           R2 Dk = s_D[k];
           R c_perp = R(0);
-          // e as the bond, k as the third atom: triplet (ti, tx, tk)
-          {
-            int tri = (ti * 2 + tx) * 2 + tk;
-            R dr = rx - rk;
+          // e as the bond, k as the third atom, triplet (ti, tx, tk); and k
+          // as the bond, e as the third atom, (ti, tk, tx): with e and k of
+          // one type the same angular function, and exponentials that are
+          // each other's reciprocals
+          const int tri = (ti * 2 + tx) * 2 + tk, trk = (ti * 2 + tk) * 2 + tx;
+          const R dr = rx - rk;
 #pragma unroll
-            for (int ll = 0; ll < 2; ++ll) {
-              R Dl = ll == 0 ? Dx.x : Dx.y;
-              R hm = P.h[tri][ll] - ct;
-              R den = P.d2[tri][ll] + hm * hm;
-              R ang = P.gam[tri][ll] * (R(1) + P.c2d2[tri][ll] * (hm * hm) / den);
-              R dang = R(-2) * P.gam[tri][ll] * P.c2[tri][ll] * hm / (den * den);
-              R ex = ct_exp<R>(P.alpha[tri][ll] * dr);
-              c_ux += Dl * P.alpha[tri][ll] * fck * ang * ex;
-              c_perp += Dl * fck * dang * ex;
+          for (int ll = 0; ll < 2; ++ll) {
+            const R De = ll == 0 ? Dx.x : Dx.y, Dl = ll == 0 ? Dk.x : Dk.y;
+            R ang, dang;
+            auto angular = [&](int t) {
+              const R hm = P.h[t][ll] - ct, hm2 = hm * hm, iden = inv(P.d2[t][ll] + hm2);
+              ang = P.gam[t][ll] * (R(1) + P.c2d2[t][ll] * (hm2 * iden));
+              dang = R(-2) * P.gam[t][ll] * P.c2[t][ll] * hm * (iden * iden);
+            };
+            angular(tri);
+            R ex = ct_exp<R>(P.alpha[tri][ll] * dr);
+            c_ux += De * P.alpha[tri][ll] * fck * ang * ex;
+            c_perp += De * fck * dang * ex;
+            if (trk != tri) {
+              angular(trk);
+              ex = ct_exp<R>(-(P.alpha[trk][ll] * dr));
+            } else {
+              ex = sizeof(R) == 8 ? inv(ex) : ct_exp<R>(-(P.alpha[trk][ll] * dr));
             }
-          }
-          // k as the bond, e as the third atom: triplet (ti, tk, tx)
-          {
-            int tri = (ti * 2 + tk) * 2 + tx;
-            R dr = rk - rx;
-#pragma unroll
-            for (int ll = 0; ll < 2; ++ll) {
-              R Dl = ll == 0 ? Dk.x : Dk.y;
-              R hm = P.h[tri][ll] - ct;
-              R den = P.d2[tri][ll] + hm * hm;
-              R ang = P.gam[tri][ll] * (R(1) + P.c2d2[tri][ll] * (hm * hm) / den);
-              R dang = R(-2) * P.gam[tri][ll] * P.c2[tri][ll] * hm / (den * den);
-              R ex = ct_exp<R>(P.alpha[tri][ll] * dr);
-              c_ux += Dl * (dfcx * ang * ex - P.alpha[tri][ll] * fcx * ang * ex);
-              c_perp += Dl * fcx * dang * ex;
-            }
+            c_ux += Dl * (dfcx * ang * ex - P.alpha[trk][ll] * fcx * ang * ex);
+            c_perp += Dl * fcx * dang * ex;
           }
           // c_perp multiplies d cos / d u_e = (u_k/r_k - cos u_e/r_e) / r_e
           R cp = c_perp * irx;
@@ -832,9 +829,9 @@ k_cov_force(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ 
 // ---------------------------------------------------------------- charge forces + gather
 // One thread per atom over its column of the list: force, per-atom energy
 // and virial in the working precision (compensated energy sum), then the
-// FP64 store, half kick, kinetic energy and per-replica sums. Threads take
-// 256-atom tiles strided over the grid, so the FP64 per-replica reductions
-// are paid once per thread, not once per atom.
+// FP64 store, half kick, kinetic energy and per-replica sums. Blocks take
+// consecutive 256-atom tiles, so the FP64 per-replica reductions are paid once
+// per thread and replica, not once per atom.
 // Blocks per SM the register allocation must allow: three for the step
 // variant at depth 4 (85 registers, no spills; 37.5% occupancy instead of
 // 25%), one elsewhere (deeper pipelines and the virial spill under a cap).
@@ -869,7 +866,9 @@ __global__ void __launch_bounds__(256, gather_min_blocks<PB, VIR>())
 #pragma unroll
     for (int k = 0; k < 10; ++k) pw[k] = R(0);
   };
-  for (int t = blockIdx.x; (long long)t * 256 < N; t += gridDim.x) {
+  int t0, t1;
+  tile_range(N, t0, t1);
+  for (int t = t0; t < t1; ++t) {
     int i = t * 256 + (int)threadIdx.x;
     if (i >= N) break;
     R4 ui = u[i];
@@ -1263,7 +1262,9 @@ void launch_bond(const DevState& S, const PotParams<R>& P, cudaStream_t st) {
 template <class R>
 static int row_lanes(const DevState& S) {
   const int full = S.nsm * (sizeof(R) == 4 ? LG_FULL32 : LG_FULL64);
-  return S.N <= S.nsm * 32 ? 32 : S.N <= full ? 8 : 1;
+  // (FP64 wants blocks of few atoms longer: rows of 70 to 240 entries in one
+  // batch left the pipe 35% busy at 6,278 atoms with 32 atoms per block)
+  return S.N <= S.nsm * (sizeof(R) == 4 ? 32 : 64) ? 32 : S.N <= full ? 8 : 1;
 }
 
 template <class R>
