@@ -470,6 +470,8 @@ static int alloc_lists(ctbop_system* s, int cap_cov, int cap_all) {
   s->alloc_cov = cap_cov;
   s->alloc_all = cap_all;
   CK(s->mixed ? plan_cg_solve<float>(S, s->off.data()) : plan_cg_solve<double>(S, s->off.data()));
+  S.Mf = nullptr;
+  if (!s->mixed && S.solver != SOLVE_LAUNCHES) CK(dalloc(s->list_buf, &S.Mf, ncol));
   return CTBOP_OK;
 }
 

@@ -30,6 +30,7 @@
 // Sums are taken in a fixed order (lanes, warps, blocks), so a solve is
 // reproducible, and every block forms the same alpha, beta and decision.
 #include <algorithm>
+#include <type_traits>
 #include <cooperative_groups.h>
 
 #include "cg.cuh"
@@ -46,6 +47,7 @@ namespace cgr = cooperative_groups;
 #define CS_GMAX 256              // groups of a cluster (CS_CLMAX * CS_W)
 #define CS_CLMAX 16              // blocks of the largest cluster
 #define CS_CL_ONE 4096           // atoms of the largest lone replica a cluster solves
+#define CS_CUT 2e-6              // how far one FP32 cycle of the FP64 policy takes the residual
 #define CS_SPIN (1 << 22)        // polls of a team barrier before it gives up (seconds)
 
 template <class R>
@@ -70,47 +72,60 @@ struct SolveArgs {
   const double* rhs;
   int* ctl;          // [4], zero between solves: maximum of the iterations, replicas done, blocks gone, arrivals
   double* part;      // [2][CS_NV][gridDim.x]: partial sums of the grid-wide team
+  int2* Mf;          // FP64 policy: the matrix once more as FP32 (j, coefficient) pairs, written by each solve
   int maxn;          // atoms of the largest replica (the cluster team's y buffers)
   int per;           // groups a block owns, at most
 };
 
 // The block inverses of a thread block's groups stay in shared memory for the
 // solve, 16 bytes of a row at a time ([group][chunk][row]: a warp reads a
-// chunk of all rows without bank conflicts).
+// chunk of all rows without bank conflicts), as FP16 (mixed policy, as they
+// are stored) or FP32 (FP64 policy: rounded alike on both sides of the
+// diagonal, so still one symmetric positive definite preconditioner).
+template <class R> struct StageType { using T = float; };
+template <> struct StageType<float> { using T = __half; };
 template <class R> struct BlockChunk {
-  using BT = typename BlockStore<R>::T;
+  using BT = typename StageType<R>::T;
   static constexpr int PER = 16 / (int)sizeof(BT);   // elements of a chunk
   static constexpr int NCH = 32 / PER;               // chunks of a row
 };
-template <class R>
-__device__ inline void stage_block(uint4* dst, const typename BlockStore<R>::T* __restrict__ binv, int i) {
-  constexpr int NCH = BlockChunk<R>::NCH;
+__device__ inline float blk_unpack(float v) { return v; }
+__device__ inline void stage_block(uint4* dst, const __half* __restrict__ binv, int i) {
   const uint4* src = reinterpret_cast<const uint4*>(binv + (size_t)(i >> 5) * 1024 + (size_t)(i & 31) * 32);
 #pragma unroll
-  for (int c = 0; c < NCH; ++c) dst[c * 32 + (i & 31)] = __ldg(src + c);
+  for (int c = 0; c < 4; ++c) dst[c * 32 + (i & 31)] = __ldg(src + c);
+}
+__device__ inline void stage_block(uint4* dst, const double* __restrict__ binv, int i) {
+  const double2* src = reinterpret_cast<const double2*>(binv + (size_t)(i >> 5) * 1024 + (size_t)(i & 31) * 32);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const double2 a = __ldg(src + 2 * c), b = __ldg(src + 2 * c + 1);
+    dst[c * 32 + (i & 31)] = make_uint4(__float_as_uint((float)a.x), __float_as_uint((float)a.y),
+                                        __float_as_uint((float)b.x), __float_as_uint((float)b.y));
+  }
 }
 // sum over chunks [c0, c1) of the lane's row times r (of the 32 atoms, in
-// shared memory)
-template <class R>
-__device__ inline R chunk_dot(const uint4* blk, const R* r, int c0, int c1) {
+// shared memory), in F
+template <class R, class F>
+__device__ inline F chunk_dot(const uint4* blk, const F* r, int c0, int c1) {
   constexpr int PER = BlockChunk<R>::PER;
-  R y = R(0);
+  F y = F(0);
 #pragma unroll 4
   for (int c = c0; c < c1; ++c) {
     union {
       uint4 v;
-      typename BlockStore<R>::T b[PER];
+      typename BlockChunk<R>::BT b[PER];
     } u;
     u.v = blk[c * 32 + (threadIdx.x & 31)];
     union {
-      uint4 v[sizeof(R) * PER / 16];
-      R x[PER];
+      uint4 v[sizeof(F) * PER / 16];
+      F x[PER];
     } w;
 #pragma unroll
-    for (int k = 0; k < (int)sizeof(R) * PER / 16; ++k)
+    for (int k = 0; k < (int)sizeof(F) * PER / 16; ++k)
       w.v[k] = reinterpret_cast<const uint4*>(r + c * PER)[k];   // (the same for all lanes)
 #pragma unroll
-    for (int k = 0; k < PER; ++k) y += (R)blk_unpack(u.b[k]) * w.x[k];
+    for (int k = 0; k < PER; ++k) y += (F)blk_unpack(u.b[k]) * w.x[k];
   }
   return y;
 }
@@ -306,11 +321,15 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double s_slots[CL ? 2 * CS_NV * CS_GMAX : 1];
   __shared__ double s_tot[CS_NV];
-  __shared__ R s_hi[3][CS_W][32], s_lo[sizeof(R) == 4 ? 3 : 1][CS_W][32];
+  __shared__ R s_hi[3][CS_W][32];
+  __shared__ float s_lo[sizeof(R) == 4 ? 3 : 1][CS_W][32];   // (compensations: FP32 sums only)
   __shared__ __align__(16) R s_r[CS_W][32];
-  __shared__ R s_abc[2];
+  __shared__ double s_abc[2];
   __shared__ int s_stop;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // the thread that forms the scalars: of the last warp, which owns no group
+  // unless the block has all it can, so its divisions run beside the update
+  const bool boss = threadIdx.x == CS_T - 32;
   Team<CL> T;
   if constexpr (CL) {
     T.rank = (int)cgr::this_cluster().block_rank();
@@ -326,8 +345,8 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
   }
   uint4* s_blk = reinterpret_cast<uint4*>(smem_raw);   // [per][chunks][32]: block inverses
   constexpr int NCH = BlockChunk<R>::NCH;
-  R* yb0 = reinterpret_cast<R*>(s_blk + (A.binv ? (size_t)A.per * NCH * 32 : 0));   // cluster team: the replica's q0,
-  R* yb1 = yb0 + A.maxn;                               // then its y, both written by every block of the cluster
+  R* yb0 = reinterpret_cast<R*>(s_blk + (A.binv ? (size_t)A.per * NCH * 32 : 0));   // cluster team: the replica's q,
+  R* yb1 = yb0 + A.maxn;                               // and its y, both written by every block of the cluster
   const int r_first = CL ? (int)(blockIdx.x / T.size) : 0, r_end = CL ? r_first + 1 : A.Rn;
   const int nh = *A.hist;
   bool alive = true;
@@ -343,77 +362,121 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
       const int g0 = a0 >> 5, ng = ((a0 + n - 1) >> 5) - g0 + 1;
       const int per = (ng + T.size - 1) / T.size;
       const int gb = min(T.rank * per, ng), G = min(gb + per, ng) - gb;
-      // slices of a row: FP64 rows are summed serially from them, at 64
-      // cycles an addition, and eight keep enough loads in flight
-      const int S = G > 0 ? min(CS_W / G, sizeof(R) == 4 ? CS_W : 8) : 0;
+      const int S = G > 0 ? CS_W / G : 0;                 // slices of a row
       const int ug = G > 0 ? warp % G : 0, us = G > 0 ? warp / G : 0;
       const bool unit = G > 0 && us < S, own = warp < G;
       const int iu = (g0 + gb + ug) * 32 + lane;          // the atom of the unit's row
       const bool inu = unit && iu >= a0 && iu < a0 + n;
       const int nau = inu ? A.nmat[iu] : 0;
       const int nwu = (int)__reduce_max_sync(CT_FULL, (unsigned)nau);
+      const int nfu = (int)__reduce_min_sync(CT_FULL, (unsigned)nau);
       const int i = (g0 + gb + warp) * 32 + lane;         // the atom this lane owns
       const bool in = own && i >= a0 && i < a0 + n;
       const MatView<R> mat(A.nl, A.M);
+      const double inv_n = 1.0 / (double)n;
       // a batch of the unit's row; past its end, zero coefficients on the
       // replica's first atom
-      const int nfu = (int)__reduce_min_sync(CT_FULL, (unsigned)nau);
-      auto fetch = [&](int e0, int (&j)[CS_B], R (&m)[CS_B]) {
+      auto entry = [&](size_t o, int& j, auto& m) {
+        if constexpr (sizeof(m) == sizeof(R)) {
+          mat.get(o, j, m);
+        } else {   // (written by this thread in the first cycle: a plain load)
+          const int2 t = A.Mf[o];
+          j = t.x;
+          m = __int_as_float(t.y);
+        }
+      };
+      auto fetch = [&](int e0, int (&j)[CS_B], auto (&m)[CS_B]) {
         const size_t o = (size_t)e0 * A.ld + iu;
         if (e0 + CS_B <= nfu) {
 #pragma unroll
-          for (int k = 0; k < CS_B; ++k) mat.get(o + (size_t)k * A.ld, j[k], m[k]);
+          for (int k = 0; k < CS_B; ++k) entry(o + (size_t)k * A.ld, j[k], m[k]);
         } else {
 #pragma unroll
           for (int k = 0; k < CS_B; ++k) {
             j[k] = a0;
-            m[k] = R(0);
-            if (e0 + k < nau) mat.get(o + (size_t)k * A.ld, j[k], m[k]);
+            m[k] = 0;
+            if (e0 + k < nau) entry(o + (size_t)k * A.ld, j[k], m[k]);
           }
         }
       };
-      // partial row sums of the unit over one vector, into s_hi/s_lo[slot]
-      auto put = [&](int slot, R hi, R lo) {
-        s_hi[slot][warp][lane] = hi;
-        if (sizeof(R) == 4) s_lo[slot][warp][lane] = lo;
+      // partial row sums of the unit over one vector, into s_hi/s_lo[slot],
+      // and the row sum of this warp's own group from them
+      auto put = [&](int slot, auto hi, auto lo) {
+        using F = decltype(hi);
+        reinterpret_cast<F(*)[32]>(&s_hi[slot][0][0])[warp][lane] = hi;
+        if (sizeof(F) == 4) s_lo[slot][warp][lane] = (float)lo;
       };
-      auto take = [&](int slot) {   // the row sum of this warp's own group
-        RowAcc<R> a;
-        R c = R(0);
-        for (int k = 0; k < S; ++k) {
-          a.add(s_hi[slot][k * G + warp][lane]);
-          if (sizeof(R) == 4) c += s_lo[slot][k * G + warp][lane];
+      auto take = [&](int slot, auto zero) {
+        using F = decltype(zero);
+        auto hi = reinterpret_cast<F(*)[32]>(&s_hi[slot][0][0]);
+        RowAcc<F> a[4];   // (four chains: the additions wait for one another)
+        F c = F(0);
+        for (int k = 0; k < S; k += 4) {
+#pragma unroll
+          for (int m = 0; m < 4; ++m)
+            if (k + m < S) {
+              a[m].add(hi[(k + m) * G + warp][lane]);
+              if (sizeof(F) == 4) c += (F)s_lo[slot][(k + m) * G + warp][lane];
+            }
         }
-        return sizeof(R) == 4 ? a.s + (a.c + c) : a.s;
+        a[0].add(a[1].s);
+        a[2].add(a[3].s);
+        a[0].add(a[2].s);
+        if (sizeof(F) == 4) c += (a[1].c + a[3].c) + a[2].c;
+        return sizeof(F) == 4 ? a[0].s + (a[0].c + c) : a[0].s;
       };
       // y = M^-1 r of the block's groups. FP32: a warp per group. FP64: a
       // group's 32 additions at 64 cycles each are shared by up to four
       // warps (one per scheduler).
       const int SA = G > 0 ? min(4, CS_W / G) : 0;
-      auto precond = [&](R r) -> R {
-        if (!A.binv) return in ? A.dinv[i] * r : R(0);
-        if (own) s_r[warp][lane] = in ? r : R(0);
-        if constexpr (sizeof(R) == 4) {
+      auto precond = [&](auto r) {
+        using F = decltype(r);
+        F* sr = reinterpret_cast<F*>(&s_r[warp][0]);
+        if (!A.binv) return in ? (F)A.dinv[i] * r : F(0);
+        if (own) sr[lane] = in ? r : F(0);
+        F y = F(0);
+        if constexpr (sizeof(F) == 4) {
           __syncwarp();
-          const R y = own ? chunk_dot<R>(s_blk + warp * NCH * 32, s_r[warp], 0, NCH) : R(0);
+          if (own) y = chunk_dot<R, F>(s_blk + warp * NCH * 32, sr, 0, NCH);
           __syncwarp();
-          return y;
         } else {
           __syncthreads();
           if (warp < SA * G)
-            s_hi[1][warp][lane] = chunk_dot<R>(s_blk + ug * NCH * 32, s_r[ug], NCH * us / SA, NCH * (us + 1) / SA);
+            s_hi[1][warp][lane] = chunk_dot<R, F>(s_blk + ug * NCH * 32, reinterpret_cast<F*>(&s_r[ug][0]),
+                                                  NCH * us / SA, NCH * (us + 1) / SA);
           __syncthreads();
-          R y = R(0);
           if (own)
             for (int k = 0; k < SA; ++k) y += s_hi[1][k * G + warp][lane];
-          return y;
+        }
+        return y;
+      };
+      if (own && A.binv) stage_block(s_blk + warp * NCH * 32, A.binv, i);
+      __syncthreads();
+      // one vector to the whole team
+      auto share = [&](R* buf, R* glob, auto v) {
+        using F = decltype(v);
+        if constexpr (CL) {
+          for (int p = 0; p < T.size; ++p) reinterpret_cast<F*>(cgr::this_cluster().map_shared_rank(buf, p))[i - a0] = v;
+        } else {
+          reinterpret_cast<F*>(glob)[i] = v;
         }
       };
-      if (own && A.binv) stage_block<R>(s_blk + warp * NCH * 32, A.binv, i);
-      __syncthreads();
       auto exchange1 = [&](double v) {   // a single FP64 sum
         const double val[1] = {own ? pair_sum(v, 0.0) : 0.0};   // (idle warps issue no FP64)
         return T.template exchange<1, false>(own, gb + warp, ng, G, val, s_tot);
+      };
+      // sums of y, r (and d) and the extremes of r over the team
+      auto exchange_y = [&](auto first, auto yi, auto ri, auto di) {
+        using F = decltype(yi);
+        constexpr int NP = decltype(first)::value ? 2 : 1;
+        double val[NP + 1] = {};
+        if (own) {
+          const F none = -F(INFINITY);
+          val[0] = (double)pair_sum(in ? yi : F(0), in ? ri : F(0));
+          if (NP == 2) val[1] = (double)pair_sum(in ? di : F(0), F(0));
+          val[NP] = (double)pair_max(in ? ri : none, in ? -ri : none);
+        }
+        return T.template exchange<NP, true>(own, gb + warp, ng, G, val, s_tot);
       };
       // ---- starting guess
       double qi = 0.0;
@@ -424,189 +487,257 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
         else if (nh == 1) qi = qo;
         A.h2[i] = x1;
         A.h1[i] = qo;
-        if constexpr (CL) {
-          for (int p = 0; p < T.size; ++p) cgr::this_cluster().map_shared_rank(yb0, p)[i - a0] = (R)qi;
-        } else {
-          A.qr[i] = (R)qi;
-        }
       }
-      if (!exchange1(qi)) { alive = false; break; }
-      const double dq0 = (cc[CG_Q] - s_tot[0]) / (double)n;
       const double mp = cc[CG_MU];
-      const double s0 = isfinite(mp) ? -mp : 0.0;
-      // ---- residual of the guess, v = H d, y = M^-1 r
-      if (unit) {
-        PartSum<R> p0, p1, p2;
-        for (int e0 = us * CS_B; e0 < nwu; e0 += S * CS_B) {
-          int j[CS_B];
-          R m[CS_B], x0[CS_B], x1[CS_B], one[CS_B];
-          fetch(e0, j, m);
-#pragma unroll
-          for (int k = 0; k < CS_B; ++k) {
-            x0[k] = CL ? yb0[j[k] - a0] : A.qr[j[k]];
-            x1[k] = A.dvec[j[k]];
-            one[k] = R(1);
-          }
-          p0.batch(m, x0);
-          p1.batch(m, x1);
-          p2.batch(m, one);
-        }
-        put(0, p0.hi(), p0.lo());
-        put(1, p1.hi(), p1.lo());
-        put(2, p2.hi(), p2.lo());
-      }
-      __syncthreads();
-      R ri = R(0), yi = R(0), di = R(0), vi = R(0), Di = R(0), pi = R(0), si = R(0), dqi = R(0);
-      auto share = [&](R val) {   // y to the whole team
-        if constexpr (CL) {
-          for (int p = 0; p < T.size; ++p) cgr::this_cluster().map_shared_rank(yb1, p)[i - a0] = val;
-        } else {
-          A.y[i] = val;
-        }
-      };
-      const R none = -R(INFINITY);
+      double shift = isfinite(mp) ? -mp : 0.0;   // subtracted from every stored r
+      double mean = 0.0, bound = 0.0, res0 = 0.0, inv_sd = 0.0;
+      R Di = R(0), di = R(0), vi = R(0), hm = R(0);
+      double chi = 0.0;
       if (in) {
         Di = A.Dg[i];
         di = A.dvec[i];
-        const R hq = take(0), hd = take(1), hm = take(2);
-        // the guess shifted by dq0: H (q0 + dq0 1) = D (q0 + dq0) + sum M q0_j + dq0 sum M
-        qi += dq0;
-        const double chi = A.rhs ? A.rhs[i] : by_type(A.T.chi, A.type[i]);
-        ri = (R)(-chi - ((double)Di * qi + (double)hq + dq0 * (double)hm) - s0);
-        vi = Di * di + hd;
+        chi = A.rhs ? A.rhs[i] : by_type(A.T.chi, A.type[i]);
       }
-      yi = precond(ri);
-      if (in) share(yi);
-      if (!in) yi = R(0);   // (a neighbouring replica's lane of a shared block)
-      {
-        double val[3] = {0.0, 0.0, 0.0};
-        if (own) {
-          val[0] = (double)pair_sum(yi, ri);
-          val[1] = (double)pair_sum(di, R(0));
-          val[2] = (double)pair_max(in ? ri : none, in ? -ri : none);
-        }
-        if (!T.template exchange<2, true>(own, gb + warp, ng, G, val, s_tot)) { alive = false; break; }
-      }
-      // ---- the iteration's scalars: thread 0 of every block forms the same
-      const double inv_n = 1.0 / (double)n, inv_sd = s_tot[2] != 0.0 ? 1.0 / s_tot[2] : 0.0;
-      double shift = s0, mean = 0.0, bound = 0.0, gp = 0.0, ap = 0.0, inv_gp = 0.0, inv_ap = 0.0, res0 = 0.0;
-      R mprev = R(0), cR = R(0);
-      auto test = [&](double sy, double sr, double hi, double lo) {
+      auto test = [&](double sy, double sr, double hi, double lo, double tol) {   // (the boss)
         mean = sr * inv_n;
         const double bh = hi - mean, bl = lo + mean;
         bound = of_key(max(key_of(bh), key_of(bl)));   // max_i |r_i - mean|
         if (!isfinite(bh) || !isfinite(bl)) bound = INFINITY;
-        s_abc[0] = (R)(sy * inv_sd);
-        s_abc[1] = (R)mean;
-        s_stop = key_of(bound) <= key_of(A.tol) ? 1 : 0;
+        s_abc[0] = sy * inv_sd;
+        s_abc[1] = mean;
+        s_stop = key_of(bound) <= key_of(tol) ? 1 : 0;
       };
-      if (threadIdx.x == 0) {
-        test(s_tot[0], s_tot[1], s_tot[4], s_tot[5]);
-        res0 = bound;
-      }
-      __syncthreads();
-      conv = s_stop;
-      cR = s_abc[0];
-      mprev = s_abc[1];
-      while (!conv && its < A.max_iter) {
-        // ---- w = H z = H y - c v, z = y - c d, and the dots r.z, w.z
+      // The CG in F from the residual ri (y = M^-1 r shared, its sums in
+      // s_abc), adding to dq, until max |r - mean| <= goal (the boss's) or
+      // the iterations are used up. Every block takes the same decisions.
+      int done = 0;
+      auto iterate = [&](auto ri, auto yi, double goal, double& dq) -> bool {
+        using F = decltype(ri);
+        const F D = (F)Di, d = (F)di, v = (F)vi;
+        F pi = F(0), si = F(0), dqi = F(0);
+        double gp = 0.0, ap = 0.0, inv_gp = 0.0, inv_ap = 0.0;
+        F cR = (F)s_abc[0], mprev = (F)s_abc[1];
+        int stop = 0;
+        const F* yb = reinterpret_cast<const F*>(yb1);
+        const F* yg = reinterpret_cast<const F*>(A.y);
+        while (!stop && its < A.max_iter) {
+          // ---- w = H z = H y - c v, z = y - c d, and the dots r.z, w.z
+          if (unit) {
+            PartSum<F> p0;
+            // the next batch is in flight while this one's y are gathered,
+            // but in the FP32 cluster team: two blocks per SM hide that
+            // latency there, and 64 registers leave no room for a second batch
+            constexpr bool AHEAD = !(CL && sizeof(R) == 4);
+            int j[CS_B];
+            F m[CS_B];
+            if (AHEAD) fetch(us * CS_B, j, m);
+            for (int e0 = us * CS_B; e0 < nwu; e0 += S * CS_B) {
+              F x0[CS_B];
+              if (!AHEAD) fetch(e0, j, m);
+#pragma unroll
+              for (int k = 0; k < CS_B; ++k) x0[k] = CL ? yb[j[k] - a0] : yg[j[k]];
+              if (AHEAD) {
+                F mc[CS_B];
+#pragma unroll
+                for (int k = 0; k < CS_B; ++k) mc[k] = m[k];
+                fetch(e0 + S * CS_B, j, m);
+                p0.batch(mc, x0);
+              } else {
+                p0.batch(m, x0);
+              }
+            }
+            put(0, p0.hi(), p0.lo());
+          }
+          __syncthreads();
+          F wi = F(0), zi = F(0);
+          double val[1] = {0.0};
+          if (own) {
+            F d0 = F(0), d1 = F(0);
+            if (in) {
+              zi = yi - cR * d;
+              wi = D * yi + take(0, F(0)) - cR * v;
+              d0 = (ri - mprev) * zi;
+              d1 = wi * zi;
+            }
+            val[0] = (double)pair_sum(d0, d1);
+          }
+          if (!T.template exchange<1, false>(own, gb + warp, ng, G, val, s_tot)) return false;
+          if (boss) {
+            // beta = g / g_prev, alpha = g / (w.z - beta g / alpha_prev)
+            const double g = s_tot[0], b = g * inv_gp;
+            double den = s_tot[1];
+            if (ap != 0.0) den -= b * g * inv_ap;
+            const double a = den != 0.0 ? g * inv(den) : 0.0;
+            s_abc[0] = a;
+            s_abc[1] = b;
+            shift += (double)mprev;   // the mean this update subtracts
+            gp = g;
+            ap = a;
+            inv_ap = den;             // (times 1 / g below)
+          }
+          __syncthreads();
+          const F a = (F)s_abc[0], b = (F)s_abc[1];
+          if (boss) {   // off the critical path: for the next beta and alpha
+            inv_gp = gp != 0.0 ? inv(gp) : 0.0;
+            inv_ap *= inv_gp;
+          }
+          if (in) {
+            pi = zi + b * pi;
+            si = wi + b * si;
+            ri = (ri - a * si) - mprev;
+            dqi += a * pi;
+          }
+          yi = precond(ri);
+          if (in) share(yb1, A.y, yi);
+          if (!exchange_y(std::false_type(), yi, ri, yi)) return false;
+          if (boss) test(s_tot[0], s_tot[1], s_tot[2], s_tot[3], goal);
+          ++its;
+          __syncthreads();
+          stop = s_stop;
+          cR = (F)s_abc[0];
+          mprev = (F)s_abc[1];
+        }
+        dq += (double)dqi;
+        done = stop;
+        return true;
+      };
+      // A cycle: the residual of q shifted onto sum q = Q, in R, then the CG
+      // from it. The mixed policy takes one, down to its tolerance. The FP64
+      // policy refines: its matrix passes are bound by the FP64 pipe, so the
+      // CG runs in FP32 on the FP64 residual, for as many digits as FP32
+      // rounding allows (CS_CUT), and the next cycle's FP64 residual decides,
+      // the one that must meet the tolerance (19,555 atoms: 756 us in 43
+      // iterations against 1,005 in 38 with the CG in FP64; the charges end
+      // nearer the minimiser than by the recursion's residual). Should a cycle gain less than a
+      // digit, the CG goes on in FP64, to the tolerance by its own recursion (a
+      // tolerance at the FP64 residual's rounding can be met that way only).
+      double last = INFINITY;
+      bool final_shift = false;
+      for (int cycle = 0;; ++cycle) {
+        if (in) share(yb0, A.qr, (R)qi);
+        if (!exchange1(qi)) { alive = false; break; }
+        const double dq0 = (cc[CG_Q] - s_tot[0]) * inv_n;
         if (unit) {
-          PartSum<R> p0;
-          // the next batch is in flight while this one's y are gathered, but
-          // in the FP32 cluster team: two blocks per SM hide that latency
-          // there, and 64 registers leave no room for a second batch
-          constexpr bool AHEAD = !(CL && sizeof(R) == 4);
-          int j[CS_B];
-          R m[CS_B];
-          if (AHEAD) fetch(us * CS_B, j, m);
-          for (int e0 = us * CS_B; e0 < nwu; e0 += S * CS_B) {
-            R x0[CS_B];
-            if (!AHEAD) fetch(e0, j, m);
+          if (cycle == 0) {   // with H d and the row sum of H for the shifts
+            PartSum<R> p0, p1, p2;
+            for (int e0 = us * CS_B; e0 < nwu; e0 += S * CS_B) {
+              int j[CS_B];
+              R m[CS_B], x0[CS_B], x1[CS_B], one[CS_B];
+              fetch(e0, j, m);
 #pragma unroll
-            for (int k = 0; k < CS_B; ++k) x0[k] = CL ? yb1[j[k] - a0] : A.y[j[k]];
-            if (AHEAD) {
-              R mc[CS_B];
+              for (int k = 0; k < CS_B; ++k) {
+                x0[k] = CL ? yb0[j[k] - a0] : A.qr[j[k]];
+                x1[k] = A.dvec[j[k]];
+                one[k] = R(1);
+                if (sizeof(R) == 8 && e0 + k < nau)
+                  A.Mf[(size_t)(e0 + k) * A.ld + iu] = make_int2(j[k], __float_as_int((float)m[k]));
+              }
+              p0.batch(m, x0);
+              p1.batch(m, x1);
+              p2.batch(m, one);
+            }
+            put(0, p0.hi(), p0.lo());
+            put(1, p1.hi(), p1.lo());
+            put(2, p2.hi(), p2.lo());
+          } else {
+            PartSum<R> p0;
+            for (int e0 = us * CS_B; e0 < nwu; e0 += S * CS_B) {
+              int j[CS_B];
+              R m[CS_B], x0[CS_B];
+              fetch(e0, j, m);
 #pragma unroll
-              for (int k = 0; k < CS_B; ++k) mc[k] = m[k];
-              fetch(e0 + S * CS_B, j, m);
-              p0.batch(mc, x0);
-            } else {
+              for (int k = 0; k < CS_B; ++k) x0[k] = CL ? yb0[j[k] - a0] : A.qr[j[k]];
               p0.batch(m, x0);
             }
+            put(0, p0.hi(), p0.lo());
           }
-          put(0, p0.hi(), p0.lo());
         }
         __syncthreads();
-        R wi = R(0), zi = R(0);
-        double val[1] = {0.0};
-        if (own) {
-          R d0 = R(0), d1 = R(0);
-          if (in) {
-            zi = yi - cR * di;
-            wi = Di * yi + take(0) - cR * vi;
-            d0 = (ri - mprev) * zi;
-            d1 = wi * zi;
-          }
-          val[0] = (double)pair_sum(d0, d1);
-        }
-        if (!T.template exchange<1, false>(own, gb + warp, ng, G, val, s_tot)) { alive = false; break; }
-        double g = 0.0;
-        if (threadIdx.x == 0) {
-          // beta = g / g_prev, alpha = g / (w.z - beta g / alpha_prev)
-          g = s_tot[0];
-          const double b = g * inv_gp;
-          double den = s_tot[1];
-          if (ap != 0.0) den -= b * g * inv_ap;
-          const bool ok = den != 0.0 && isfinite(den);
-          const double id = ok ? recip(den) : 0.0;
-          const double a = ok ? g * id : (den == 0.0 ? 0.0 : g / den);
-          s_abc[0] = (R)a;
-          s_abc[1] = (R)b;
-          shift += (double)mprev;   // the mean this update subtracts
-          gp = g;
-          ap = a;
-          inv_ap = den;             // (times 1 / g below)
-        }
-        __syncthreads();
-        const R a = s_abc[0], b = s_abc[1];
+        R ri = R(0);
         if (in) {
-          pi = zi + b * pi;
-          si = wi + b * si;
-          ri = (ri - a * si) - mprev;
-          dqi += a * pi;
-        }
-        yi = precond(ri);
-        if (in) share(yi);
-        if (!in) yi = R(0);
-        {
-          double v2[2] = {0.0, 0.0};
-          if (own) {
-            v2[0] = (double)pair_sum(yi, ri);
-            v2[1] = (double)pair_max(in ? ri : none, in ? -ri : none);
+          const R hq = take(0, R(0));
+          if (cycle == 0) {
+            vi = Di * di + take(1, R(0));
+            hm = take(2, R(0));
           }
-          if (!T.template exchange<1, true>(own, gb + warp, ng, G, v2, s_tot)) { alive = false; break; }
+          // q shifted by dq0: H (q + dq0 1) = D (q + dq0) + sum M q_j + dq0 sum M
+          qi += dq0;
+          ri = (R)(-chi - ((double)Di * qi + (double)hq + dq0 * (double)hm) - shift);
         }
-        if (threadIdx.x == 0) test(s_tot[0], s_tot[1], s_tot[2], s_tot[3]);
-        ++its;
+        // (FP32: what the CG starts from; every block's `shift` is the boss's)
+        float yf = precond((float)ri);
+        if (in) share(yb1, A.y, yf);
+        const bool ok = cycle == 0 ? exchange_y(std::true_type(), (R)yf, ri, di) : exchange_y(std::false_type(), (R)yf, ri, di);
+        if (!ok) { alive = false; break; }
+        if (boss) {
+          if (cycle == 0) {
+            inv_sd = s_tot[2] != 0.0 ? 1.0 / s_tot[2] : 0.0;
+            test(s_tot[0], s_tot[1], s_tot[4], s_tot[5], A.tol);
+            res0 = bound;
+          } else {
+            test(s_tot[0], s_tot[1], s_tot[2], s_tot[3], A.tol);
+          }
+        }
         __syncthreads();
         conv = s_stop;
-        cR = s_abc[0];
-        mprev = s_abc[1];
-        if (threadIdx.x == 0) {   // off the critical path: for the next beta and alpha
-          inv_gp = gp != 0.0 && isfinite(gp) ? recip(gp) : (gp == 0.0 ? 0.0 : 1.0 / gp);
-          inv_ap *= inv_gp;
+        if (conv || its >= A.max_iter) break;   // (uniform)
+        double dq = 0.0;
+        bool go;
+        if constexpr (sizeof(R) == 4) {
+          go = iterate(ri, yf, A.tol, dq);
+          qi += dq;
+          conv = done;
+          final_shift = true;
+          if (!go) alive = false;
+          break;
+        } else {
+          // the boss knows the residual; whether it fell tenfold, for all
+          if (boss) {
+            s_stop = bound <= 0.1 * last ? 1 : 0;
+            last = bound;
+          }
+          __syncthreads();
+          const bool fell = s_stop != 0;
+          if (fell) {
+            go = iterate((float)ri, yf, fmax(0.3 * A.tol, bound * CS_CUT), dq);
+          } else {
+            const double yd = precond((double)ri);
+            if (in) share(yb1, A.y, yd);
+            go = exchange_y(std::false_type(), yd, ri, yd);
+            if (go) {
+              if (boss) test(s_tot[0], s_tot[1], s_tot[2], s_tot[3], A.tol);
+              __syncthreads();
+              go = iterate((double)ri, yd, A.tol, dq);
+            }
+          }
+          qi += dq;
+          if (!go) { alive = false; break; }
+          if (!fell) {
+            conv = done;
+            final_shift = true;
+            break;
+          }
+          // the mean is part of the shift from here on (the boss's, to all)
+          if (boss) {
+            shift += mean;
+            s_abc[0] = shift;
+          }
+          __syncthreads();
+          shift = s_abc[0];
+          __syncthreads();
         }
       }
       if (!alive) break;
-      // ---- q <- q + dq, shifted onto sum q = Q
-      double qt = in ? qi + (double)dqi : 0.0;
-      if (!exchange1(qt)) { alive = false; break; }
-      if (in) {
-        qt += (cc[CG_Q] - s_tot[0]) / (double)n;
-        A.q[i] = qt;
-        A.qr[i] = (R)qt;
+      // ---- the charges, after a CG in R once more onto sum q = Q
+      if (final_shift) {
+        if (!exchange1(qi)) { alive = false; break; }
+        qi += (cc[CG_Q] - s_tot[0]) * inv_n;
       }
-      if (T.rank == 0 && threadIdx.x == 0) {
+      if (in) {
+        A.q[i] = qi;
+        A.qr[i] = (R)qi;
+      }
+      if (T.rank == 0 && boss) {
         cc[CG_M] = mean;
         cc[CG_SHIFT] = shift;
         cc[CG_RESMAX] = bound;
@@ -646,7 +777,7 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
 // cluster team's two vectors.
 template <class R, bool CL>
 static size_t solve_smem(int per, int maxn, int precond) {
-  return (precond ? (size_t)per * 1024 * sizeof(typename BlockStore<R>::T) : 0) + (CL ? 2 * (size_t)maxn * sizeof(R) : 0);
+  return (precond ? (size_t)per * 1024 * sizeof(typename BlockChunk<R>::BT) : 0) + (CL ? 2 * (size_t)maxn * sizeof(R) : 0);
 }
 
 template <class R, bool CL>
@@ -684,7 +815,7 @@ cudaError_t launch_cg_solve(const DevState& S, const TypeParams& T, double tol, 
   A.qr = (R*)S.qr; A.y = (R*)S.cy;
   A.cg = S.cg; A.conv = S.cg_conv; A.iters = S.cg_iters; A.it = S.cg_it; A.hist = S.cg_hist; A.total = S.cg_total;
   A.err = S.err; A.tol = tol; A.max_iter = max_iter; A.rhs = rhs;
-  A.ctl = S.solve_ctl; A.part = S.solve_part; A.maxn = S.solve_maxn; A.per = S.solve_per;
+  A.ctl = S.solve_ctl; A.part = S.solve_part; A.maxn = S.solve_maxn; A.per = S.solve_per; A.Mf = S.Mf;
   return S.solver == SOLVE_CLUSTER ? launch_solve<R, true>(S, A, st) : launch_solve<R, false>(S, A, st);
 }
 
@@ -702,10 +833,11 @@ cudaError_t launch_cg_solve(const DevState& S, const TypeParams& T, double tol, 
 //     1.25 million atoms 0.57 ms against 0.33;
 //   * one larger replica whose matrix fits L2: the grid-wide team;
 //   * anything else: the per-iteration kernels.
-// Solve times, microseconds per MD step before (launches) and with this
-// kernel: FP64, 64 atoms 1,000 -> 170 (18 iterations), 512 atoms 1,950 -> 290
-// (31), 19,555 atoms 2,820 -> 1,000 (38); mixed, 11,491 atoms 520 -> 160 (11),
-// 32 configurations of 64-512 atoms 840 -> 140 (20).
+// Solve times, microseconds per MD step by launches and with this kernel:
+// FP64, 64 atoms 1,000 -> 149 (18 -> 21 iterations, see k_cg_solve's cycles),
+// 512 atoms 1,950 -> 240 (31 -> 34), 19,555 atoms 2,820 -> 756 (38 -> 43);
+// mixed, 11,491 atoms 520 -> 160 (11), 32 configurations of 64-512 atoms
+// 840 -> 140 (20).
 template <class R>
 cudaError_t plan_cg_solve(DevState& S, const int64_t* off) {
   S.solver = SOLVE_LAUNCHES;

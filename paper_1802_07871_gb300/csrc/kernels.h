@@ -114,6 +114,7 @@ struct DevState {
   void* stiff_pe = nullptr;     // double2 [N * cap_cov]
   void* bo = nullptr;           // Real4[N*cap_cov]
   void* gslot = nullptr;        // Real4[N*cap_cov]
+  int2* Mf = nullptr;           // FP64 policy, whole-solve kernel: [cap_all*ld] FP32 (j, coefficient) pairs of M
   void* M = nullptr;            // [cap_all*ld] charge matrix: FP32 (j, coefficient) int2 pairs, or FP64 coefficients
   void *Dg = nullptr, *dinv = nullptr;   // Real[N]: Hessian diagonal without self-images, Jacobi inverse
   // CG: the iterate is q itself (FP64); the rest in the working precision
