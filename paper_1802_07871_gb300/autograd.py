@@ -21,8 +21,15 @@ class Energy(torch.autograd.Function):
         xd = x.detach().to(torch.float64).contiguous()
         system.set_positions(xd.cpu().numpy() if not xd.is_cuda else xd)
         system.compute()
-        E = torch.as_tensor(system.get("energy"), dtype=x.dtype, device=x.device)
-        F = torch.as_tensor(system.get("forces"), dtype=x.dtype, device=x.device)
+        if x.is_cuda and system.ordered_with_current_stream():
+            E = torch.empty(system.R, dtype=torch.float64, device=x.device)
+            F = torch.empty((system.n, 3), dtype=torch.float64, device=x.device)
+            system.get("energy", out=E)
+            system.get("forces", out=F)
+            E, F = E.to(x.dtype), F.to(x.dtype)
+        else:
+            E = torch.as_tensor(system.get("energy"), dtype=x.dtype, device=x.device)
+            F = torch.as_tensor(system.get("forces"), dtype=x.dtype, device=x.device)
         ctx.save_for_backward(F)
         ctx.rep = torch.as_tensor(system.replica_index(), device=x.device)
         return E

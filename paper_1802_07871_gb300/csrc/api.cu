@@ -102,6 +102,7 @@ struct ctbop_system {
   float build_ms[BUILD_SHAPES] = {};
   bool tune_pending = false;
   double g_step_dt = -1.0;
+  bool eval_seen = false;       // an evaluation ran since the graphs were last dropped
   bool use_graph = true;
   // pinned host scratch
   int* h_int = nullptr;
@@ -224,6 +225,7 @@ static void destroy_graphs(ctbop_system* s) {
   if (s->g_step) cudaGraphExecDestroy(s->g_step);
   s->g_eval = s->g_step = nullptr;
   s->g_step_dt = -1.0;
+  s->eval_seen = false;
 }
 
 static int setup_reps(ctbop_system* s) {
@@ -385,7 +387,8 @@ static int alloc_atoms(ctbop_system* s) {
   CK(dalloc(s->rep_buf, &S.rebuild_count, 1));
   CK(dalloc(s->rep_buf, &S.precond_epoch, 1));
   CK(cudaMemsetAsync(S.precond_epoch, 0xff, sizeof(long long), s->stream));   // -1: form at the first solve
-  CK(dalloc(s->rep_buf, &S.maxcnt, 3));
+  CK(dalloc(s->rep_buf, &S.maxcnt, 4));   // and the error word, read back together
+  S.err = reinterpret_cast<unsigned*>(S.maxcnt + 3);
   CK(dalloc(s->rep_buf, &S.stiff_n, 1));
   CK(zero_async(s, S.stiff_n, sizeof(int)));
   CK(dalloc(s->rep_buf, &S.acc_mode, (size_t)s->R));
@@ -398,7 +401,6 @@ static int alloc_atoms(ctbop_system* s) {
     CK(dalloc(s->atom_buf, &u64, (size_t)std::max(N, 1) * 32));
     S.u64 = u64;
   }
-  CK(dalloc(s->rep_buf, &S.err, 1));
   CK(dalloc(s->rep_buf, &S.cg_it, 1));
   CK(dalloc(s->rep_buf, &S.cg_blocks, 3));
   CK(dalloc(s->rep_buf, &S.cg_hist, 1));
@@ -612,7 +614,6 @@ static int read_err(ctbop_system* s, unsigned& bits) {
 // them and builds again.
 static int ensure_lists(ctbop_system* s) {
   DevState& S = s->S;
-  int one = 1;
   if (!s->caps_known) {
     int cc = s->o.cap_cov > 0 ? s->o.cap_cov : 32;
     int ca = s->o.cap_all > 0 ? s->o.cap_all : 64;
@@ -621,16 +622,17 @@ static int ensure_lists(ctbop_system* s) {
   }
   for (int attempt = 0;; ++attempt) {
     if (attempt > 4) return fail(s, CTBOP_ERR_NEIGH_OVERFLOW, "could not size the neighbour lists");
-    CK(cudaMemcpyAsync(S.flag_rebuild, &one, sizeof(int), cudaMemcpyHostToDevice, s->stream));
+    CK(cudaMemsetAsync(S.flag_rebuild, 1, sizeof(int), s->stream));   // (any non-zero word)
     CK(cudaMemsetAsync(S.err, 0, sizeof(unsigned), s->stream));
     if (s->mixed) launch_rebuild<float>(S, s->Pf, s->stream);
     else launch_rebuild<double>(S, s->Pd, s->stream);
     CK(cudaGetLastError());
-    unsigned bits = 0;
-    int rc = read_err(s, bits);
-    if (rc) return rc;
-    int mc[3];
-    CK(sync_copy(s, mc, S.maxcnt, sizeof(mc), cudaMemcpyDeviceToHost));
+    // the counts and the error word in one read
+    CK(cudaMemcpyAsync(s->h_int, S.maxcnt, 4 * sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    CK(cudaStreamSynchronize(s->stream));
+    const int mc[3] = {s->h_int[0], s->h_int[1], s->h_int[2]};
+    const unsigned bits = (unsigned)s->h_int[3];
+    int rc = CTBOP_OK;
     if (bits & CT_ERR_NONFINITE) return fail(s, CTBOP_ERR_NONFINITE, "non-finite position");
     bool over = (bits & (CT_ERR_NBR_OVERFLOW | CT_ERR_COV_OVERFLOW)) != 0;
     if (!over && (bits & CT_ERR_REV_MISSING)) return fail(s, CTBOP_ERR_CUDA, "internal: asymmetric covalent list");
@@ -742,7 +744,14 @@ static int eval_t(ctbop_system* s, const PotParams<Rr>& P, uint32_t flags) {
     s->virial_stale = false;
     return CTBOP_OK;
   }
-  if (s->use_graph && solve) {
+  // a graph is worth its capture from the second evaluation on: a program that
+  // sets parameters or boxes before each evaluation would capture every time
+  // (a host-polled loop of launches would cost it more). 32 configurations with
+  // new positions and gradients through autograd: 2.99 ms a pass with the capture
+  // and results through the host, 2.52 ms without
+  const bool direct = !s->g_eval && !s->eval_seen && s->S.solver != SOLVE_LAUNCHES;
+  if (solve) s->eval_seen = true;
+  if (s->use_graph && solve && !direct) {
     if (!s->g_eval) {
       int rc = capture_graph<Rr>(s, P, false, 0.0, &s->g_eval);
       if (rc) return rc;
@@ -1810,29 +1819,35 @@ int ctbop_minimize(ctbop_system* s, int64_t max_iter, double fmax, double dt0, d
   CK(zero_async(s, S.v, sizeof(double) * 3 * (size_t)S.N));   // from rest
   const double half_skin2 = 0.25 * s->o.skin * s->o.skin;
   int redo = 0;
+  bool moved = false;   // an evaluation of this call is behind the error word
   for (;;) {
-    launch_fire_reduce(S, fire, cfg, ctl, ctl + 1, s->stream);
+    // (leaves the states alone after an evaluation whose lists overflowed)
+    launch_fire_reduce(S, fire, cfg, ctl, ctl + 1, moved ? S.err : nullptr, s->stream);
     CK(cudaGetLastError());
-    CK(sync_copy(s, s->h_int, ctl + 1, sizeof(int), cudaMemcpyDeviceToHost));
-    if (*s->h_int == 0) break;
-    if (s->mixed) launch_fire_move<float>(S, s->T, fire, half_skin2, s->stream);
-    else launch_fire_move<double>(S, s->T, fire, half_skin2, s->stream);
-    CK(cudaGetLastError());
-    CK(zero_async(s, S.err, sizeof(unsigned)));
-    rc = ctbop_compute(s, 0);
-    unsigned bits = 0;
-    if (!rc) rc = read_err(s, bits);
-    while (!rc && (bits & (CT_ERR_NBR_OVERFLOW | CT_ERR_COV_OVERFLOW))) {
+    CK(cudaMemcpyAsync(s->h_int, ctl + 1, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    CK(cudaMemcpyAsync(s->h_int + 1, S.err, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
+    CK(cudaStreamSynchronize(s->stream));
+    const unsigned bits = moved ? (unsigned)s->h_int[1] : 0u;
+    if (bits & (CT_ERR_NBR_OVERFLOW | CT_ERR_COV_OVERFLOW)) {
       if (++redo > 3) {
         rc = fail(s, CTBOP_ERR_NEIGH_OVERFLOW, "neighbour lists kept overflowing");
         break;
       }
       rc = regrow_and_recompute(s);
-      if (!rc) rc = read_err(s, bits);
+      if (rc) break;
+      continue;
     }
-    if (!rc && (bits & CT_ERR_NONFINITE)) rc = fail(s, CTBOP_ERR_NONFINITE, "non-finite energy, force or position");
+    if (bits & CT_ERR_NONFINITE) rc = fail(s, CTBOP_ERR_NONFINITE, "non-finite energy, force or position");
+    if (!rc && (bits & CT_ERR_SOLVER)) rc = fail(s, CTBOP_ERR_CUDA, "internal: the charge solve gave up waiting");
     if (!rc && (bits & CT_ERR_CG_MAXITER)) rc = fail(s, CTBOP_ERR_CG_NOT_CONVERGED, "charge CG reached max_iter");
+    if (rc || *s->h_int == 0) break;
+    if (s->mixed) launch_fire_move<float>(S, s->T, fire, half_skin2, s->stream);
+    else launch_fire_move<double>(S, s->T, fire, half_skin2, s->stream);
+    CK(cudaGetLastError());
+    CK(zero_async(s, S.err, sizeof(unsigned)));
+    rc = ctbop_compute(s, 0);
     if (rc) break;
+    moved = true;
   }
   if (!rc) {
     CK(sync_copy(s, fh.data(), fire, sizeof(double) * fh.size(), cudaMemcpyDeviceToHost));

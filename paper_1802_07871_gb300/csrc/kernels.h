@@ -237,8 +237,10 @@ enum FireSlots {
 struct FireCfg {
   double fmax2, dt_max, f_inc, f_dec, alpha0, f_alpha, n_min, max_iter;
 };
+// (err: the error word of the evaluation to judge, or null; list overflows
+// leave the states alone)
 void launch_fire_reduce(const DevState& S, double* fire, const FireCfg& cfg, int* blocks, int* active,
-                        cudaStream_t st);
+                        const unsigned* err, cudaStream_t st);
 template <class R>
 void launch_fire_move(const DevState& S, const TypeParams& T, const double* fire, double half_skin2,
                       cudaStream_t st);

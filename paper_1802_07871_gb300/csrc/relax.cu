@@ -16,7 +16,8 @@ namespace ct {
 __global__ void k_fire_reduce(int N, int R, const int* __restrict__ rep, const uint8_t* __restrict__ frozen,
                               const double* __restrict__ F, const double* __restrict__ v,
                               double* __restrict__ fire, FireCfg cfg, int* __restrict__ blocks,
-                              int* __restrict__ active) {
+                              int* __restrict__ active, const unsigned* __restrict__ err) {
+  if (err && (*err & (CT_ERR_NBR_OVERFLOW | CT_ERR_COV_OVERFLOW))) return;   // (forces of cut lists: the host grows them first)
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   RepAcc<3> acc;
   acc.init();
@@ -125,9 +126,9 @@ __global__ void k_fire_move(int N, double half_skin2, const int* __restrict__ ty
 }
 
 void launch_fire_reduce(const DevState& S, double* fire, const FireCfg& cfg, int* blocks, int* active,
-                        cudaStream_t st) {
+                        const unsigned* err, cudaStream_t st) {
   int n = S.N > 0 ? S.N : 1;
-  k_fire_reduce<<<(n + 255) / 256, 256, 0, st>>>(S.N, S.R, S.rep, S.frozen, S.F, S.v, fire, cfg, blocks, active);
+  k_fire_reduce<<<(n + 255) / 256, 256, 0, st>>>(S.N, S.R, S.rep, S.frozen, S.F, S.v, fire, cfg, blocks, active, err);
 }
 
 template <class R>

@@ -321,6 +321,7 @@ class System:
         self.R = 0
         self.precision = precision
         self.device = device
+        self._stream = 0
 
     def _check(self, rc, what):
         if rc != OK:
@@ -341,6 +342,14 @@ class System:
     # ---- setup
     def set_stream(self, stream_handle: int):
         self._check(self._L.ctbop_set_stream(self._h, C.c_void_p(stream_handle)), "set_stream")
+        self._stream = int(stream_handle or 0)
+
+    def ordered_with_current_stream(self) -> bool:
+        """Whether work on torch's current stream of this system's device is
+        ordered with the system's: the same stream, or the default stream
+        against the library's own (which synchronises with it)."""
+        import torch
+        return torch.cuda.current_stream(self.device).cuda_stream == self._stream
 
     def set_params_struct(self, P: Params):
         """Replace the parameters from a filled struct (e.g. one built from a
