@@ -1484,36 +1484,39 @@ static int param_grad_impl(ctbop_system* s, const double* w_E, const double* E_r
   const bool fp32 = sizeof(Rr) == 4;
   int rc = ctbop_compute(s, 0);
   if (rc) return rc;
-  std::vector<double> E(R), F((size_t)3 * N);
-  CK(cudaMemcpy2DAsync(E.data(), 8, S.rep_acc + RA_E, RA_STRIDE * 8, 8, R, cudaMemcpyDeviceToHost, st));
-  CK(sync_copy(s, F.data(), S.F, sizeof(double) * 3 * N, cudaMemcpyDeviceToHost));
-  // loss and its derivatives with respect to E_r and F_i
-  double loss = 0.0;
-  std::vector<double> a(R, 0.0), g((size_t)3 * N, 0.0), one(R, 1.0);
-  double gmax = 0.0;
-  for (int r = 0; r < R; ++r) {
-    if (w_E && E_ref) {
+  double *d_w = nullptr, *d_one = nullptr, *d_g = nullptr, *d_dir = nullptr, *d_v = nullptr, *d_cg = nullptr;
+  double *d_h1 = nullptr, *d_h2 = nullptr, *d_q0 = nullptr, *d_lam = nullptr, *d_l = nullptr, *d_out = nullptr;
+  double *d_wF = nullptr, *d_Fref = nullptr;
+  int* d_hist = nullptr;
+  const bool forces = w_F && F_ref;
+  Scratch scr(st, s->pool);
+  if (scr.alloc(&d_w, R) || scr.alloc(&d_one, R) || scr.alloc(&d_g, 2 * PG_NPARAM) || scr.alloc(&d_l, 2 * PG_NPARAM) ||
+      scr.alloc(&d_dir, (size_t)3 * N) || scr.alloc(&d_v, N) || scr.alloc(&d_cg, (size_t)R * CG_STRIDE) ||
+      scr.alloc(&d_h1, N) || scr.alloc(&d_h2, N) || scr.alloc(&d_q0, N) || scr.alloc(&d_lam, N) ||
+      scr.alloc(&d_out, (size_t)R + 3) || scr.alloc(&d_hist, 1) ||
+      (forces && (scr.alloc(&d_wF, R) || scr.alloc(&d_Fref, (size_t)3 * N))))
+    return fail(s, CTBOP_ERR_OOM, "param_grad: temporary buffers");
+  // loss and its derivatives with respect to F_i (device) and E_r (host): the
+  // energies, the force part of the loss and max |g| come back in one read
+  CK(zero_async(s, d_out + R, 3 * sizeof(double)));
+  if (forces) {
+    CK(cudaMemcpyAsync(d_wF, w_F, sizeof(double) * R, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(d_Fref, F_ref, sizeof(double) * 3 * (size_t)N, cudaMemcpyHostToDevice, st));
+    launch_force_residual(S, d_Fref, s->ordered ? s->d_order : nullptr, d_wF, d_dir, d_out + R, st);
+  }
+  CK(cudaMemcpy2DAsync(d_out, 8, S.rep_acc + RA_E, RA_STRIDE * 8, 8, R, cudaMemcpyDeviceToDevice, st));
+  std::vector<double> E((size_t)R + 2);
+  CK(sync_copy(s, E.data(), d_out, sizeof(double) * E.size(), cudaMemcpyDeviceToHost));
+  double loss = E[R];
+  const double gmax = E[R + 1];
+  std::vector<double> a(R, 0.0), one(R, 1.0);
+  if (w_E && E_ref)
+    for (int r = 0; r < R; ++r) {
       double d = E[r] - E_ref[r];
       loss += w_E[r] * d * d;
       a[r] = 2.0 * w_E[r] * d;
     }
-    if (w_F && F_ref)
-      for (int64_t i = s->off[r]; i < s->off[r + 1]; ++i)
-        for (int k = 0; k < 3; ++k) {
-          double d = F[3 * i + k] - F_ref[3 * i + k];
-          loss += w_F[r] * d * d;
-          g[3 * i + k] = 2.0 * w_F[r] * d;
-          gmax = std::max(gmax, std::fabs(g[3 * i + k]));
-        }
-  }
   *loss_out = loss;
-  double *d_w = nullptr, *d_one = nullptr, *d_g = nullptr, *d_dir = nullptr, *d_v = nullptr, *d_cg = nullptr;
-  double *d_h1 = nullptr, *d_h2 = nullptr, *d_q0 = nullptr, *d_lam = nullptr;
-  Scratch scr(st, s->pool);
-  if (scr.alloc(&d_w, R) || scr.alloc(&d_one, R) || scr.alloc(&d_g, 2 * PG_NPARAM) ||
-      scr.alloc(&d_dir, (size_t)3 * N) || scr.alloc(&d_v, N) || scr.alloc(&d_cg, (size_t)R * CG_STRIDE) ||
-      scr.alloc(&d_h1, N) || scr.alloc(&d_h2, N) || scr.alloc(&d_q0, N) || scr.alloc(&d_lam, N))
-    return fail(s, CTBOP_ERR_OOM, "param_grad: temporary buffers");
   const ctbop_params& P = s->p;
   std::vector<double> G(2 * PG_NPARAM, 0.0), L(2 * PG_NPARAM, 0.0);
   CK(cudaMemcpyAsync(d_w, a.data(), sizeof(double) * R, cudaMemcpyHostToDevice, st));
@@ -1525,48 +1528,32 @@ static int param_grad_impl(ctbop_system* s, const double* w_E, const double* E_r
     CK(cudaStreamSynchronize(st));
   } else {
     // energy part, T1 and v in one forward-mode pass along g
-    std::vector<double> v(N);
-    CK(cudaMemcpyAsync(d_dir, g.data(), sizeof(double) * 3 * N, cudaMemcpyHostToDevice, st));
     CK(launch_param_grad(S, P, fp32, d_w, d_one, d_dir, nullptr, d_g, d_v, st));
-    CK(cudaMemcpyAsync(G.data(), d_g, sizeof(double) * 2 * PG_NPARAM, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(v.data(), d_v, sizeof(double) * N, cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    for (int k = 0; k < PG_NPARAM; ++k) G[k] -= G[PG_NPARAM + k];
-    // rhs of the solver's H q + chi = mu 1 form: chi := -v (the matrix at x
-    // is the one the charge solve above assembled)
-    double vmax = 0.0;
-    for (int i = 0; i < N; ++i) {
-      v[i] = -v[i];
-      vmax = std::max(vmax, std::fabs(v[i]));
-    }
-    CK(cudaMemcpyAsync(d_v, v.data(), sizeof(double) * N, cudaMemcpyHostToDevice, st));
     // keep the charges and the solver state: per-replica scalars, history
     CK(cudaMemcpyAsync(d_q0, S.q, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
     CK(cudaMemcpyAsync(d_cg, S.cg, sizeof(double) * R * CG_STRIDE, cudaMemcpyDeviceToDevice, st));
     CK(cudaMemcpyAsync(d_h1, S.cqh1, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
     CK(cudaMemcpyAsync(d_h2, S.cqh2, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
-    int hist_saved = 0;
-    CK(sync_copy(s, &hist_saved, S.cg_hist, sizeof(int), cudaMemcpyDeviceToHost));
-    // the adjoint: zero total per replica, cold start
-    std::vector<double> cgh((size_t)R * CG_STRIDE);
-    CK(sync_copy(s, cgh.data(), S.cg, sizeof(double) * cgh.size(), cudaMemcpyDeviceToHost));
-    for (int r = 0; r < R; ++r) cgh[(size_t)r * CG_STRIDE + CG_Q] = 0.0;
-    CK(sync_copy(s, S.cg, cgh.data(), sizeof(double) * cgh.size(), cudaMemcpyHostToDevice));
-    int zero = 0;
-    CK(sync_copy(s, S.cg_hist, &zero, sizeof(int), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(d_hist, S.cg_hist, sizeof(int), cudaMemcpyDeviceToDevice, st));
+    // rhs of the solver's H q + chi = mu 1 form: chi := -v (the matrix at x
+    // is the one the charge solve above assembled); zero total per replica,
+    // cold start
+    launch_adjoint_rhs(S, d_v, d_out + R + 2, st);
+    CK(cudaGetLastError());
     // FP64: the charge solve's absolute tolerance. FP32: the charge solve's
     // relative reach (its tolerance over the electronegativity scale, about
     // 2e-6) applied to the size of this right-hand side.
     double tol = cg_tol(s);
-    if (fp32 && s->o.cg_tol <= 0) tol = std::max(tol, 2e-6 * vmax);
+    if (fp32 && s->o.cg_tol <= 0) {
+      double vmax = 0.0;
+      CK(sync_copy(s, &vmax, d_out + R + 2, sizeof(double), cudaMemcpyDeviceToHost));
+      tol = std::max(tol, 2e-6 * vmax);
+    }
     SolveCfg cfg{tol, s->o.cg_max_iter, 0, 0};
     if (S.solver == SOLVE_LAUNCHES) launch_cg_begin<Rr>(S, s->T, st, cfg.tol, d_v);
     rc = solve_direct<Rr>(s, cfg, d_v, st);
     if (rc) return rc;
     if (S.solver == SOLVE_LAUNCHES) launch_cg_end<Rr>(S, st);
-    unsigned bits = 0;
-    rc = read_err(s, bits);
-    if (!rc && (bits & CT_ERR_CG_MAXITER)) rc = fail(s, CTBOP_ERR_CG_NOT_CONVERGED, "param_grad: adjoint CG reached max_iter");
     // lambda out, the charges and the solver state back
     CK(cudaMemcpyAsync(d_lam, S.q, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
     CK(cudaMemcpyAsync(S.q, d_q0, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
@@ -1574,15 +1561,17 @@ static int param_grad_impl(ctbop_system* s, const double* w_E, const double* E_r
     CK(cudaMemcpyAsync(S.cg, d_cg, sizeof(double) * R * CG_STRIDE, cudaMemcpyDeviceToDevice, st));
     CK(cudaMemcpyAsync(S.cqh1, d_h1, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
     CK(cudaMemcpyAsync(S.cqh2, d_h2, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
-    CK(cudaMemcpyAsync(S.cg_hist, &hist_saved, sizeof(int), cudaMemcpyHostToDevice, st));
-    if (!rc) {
-      // lambda . d(Hq + chi)/dtheta: forward mode along the charges
-      CK(launch_param_grad(S, P, fp32, d_one, d_one, nullptr, d_lam, d_g, nullptr, st));
-      CK(cudaMemcpyAsync(L.data(), d_g, sizeof(double) * 2 * PG_NPARAM, cudaMemcpyDeviceToHost, st));
-    }
+    CK(cudaMemcpyAsync(S.cg_hist, d_hist, sizeof(int), cudaMemcpyDeviceToDevice, st));
+    // lambda . d(Hq + chi)/dtheta: forward mode along the charges
+    CK(launch_param_grad(S, P, fp32, d_one, d_one, nullptr, d_lam, d_l, nullptr, st));
+    CK(cudaMemcpyAsync(s->h_int, S.err, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(G.data(), d_g, sizeof(double) * 2 * PG_NPARAM, cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(L.data(), d_l, sizeof(double) * 2 * PG_NPARAM, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    if (!rc)
-      for (int k = 0; k < PG_NPARAM; ++k) G[k] += L[PG_NPARAM + k];
+    const unsigned bits = (unsigned)*s->h_int;
+    if (bits & CT_ERR_SOLVER) rc = fail(s, CTBOP_ERR_CUDA, "internal: the charge solve gave up waiting");
+    if (!rc && (bits & CT_ERR_CG_MAXITER)) rc = fail(s, CTBOP_ERR_CG_NOT_CONVERGED, "param_grad: adjoint CG reached max_iter");
+    for (int k = 0; k < PG_NPARAM; ++k) G[k] += L[PG_NPARAM + k] - G[PG_NPARAM + k];
   }
   if (rc) return rc;
   G[PG_MASS] = G[PG_MASS + 1] = 0.0;   // the mass is not in E
@@ -1605,13 +1594,6 @@ int ctbop_param_grad(ctbop_system* s, const double* w_E, const double* E_ref, co
   static_assert(offsetof(ctbop_params, E0) == PG_E0 * sizeof(double), "layout");
   static_assert(offsetof(ctbop_params, k_e) == PG_KE * sizeof(double), "layout");
   double* out = reinterpret_cast<double*>(dtheta);
-  std::vector<double> Fs;
-  if (F_ref && s->ordered) {   // the targets in storage order
-    Fs.resize((size_t)3 * s->S.N);
-    for (int64_t k = 0; k < s->S.N; ++k)
-      for (int d = 0; d < 3; ++d) Fs[3 * k + d] = F_ref[3 * s->order[k] + d];
-    F_ref = Fs.data();
-  }
   return s->mixed ? param_grad_impl<float>(s, w_E, E_ref, w_F, F_ref, loss, out)
                   : param_grad_impl<double>(s, w_E, E_ref, w_F, F_ref, loss, out);
 }

@@ -629,7 +629,70 @@ __global__ void __launch_bounds__(PC_T)
   }
 }
 
+// The force part of the loss and its derivative with respect to the forces.
+__global__ void k_force_residual(int N, const double* __restrict__ F, const double* __restrict__ F_ref,
+                                 const int* __restrict__ order, const int* __restrict__ rep,
+                                 const double* __restrict__ wF, double* __restrict__ g, double* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  double loss = 0.0, m = 0.0;
+  if (i < N) {
+    const size_t k = order ? (size_t)order[i] : (size_t)i;
+    const double w = wF[rep[i]];
+    double d2 = 0.0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double d = F[3 * (size_t)i + c] - F_ref[3 * k + c], gi = 2.0 * w * d;
+      g[3 * (size_t)i + c] = gi;
+      m = fmax(m, fabs(gi));
+      d2 += d * d;
+    }
+    loss = w * d2;
+  }
+  loss = warp_sum(loss);
+  m = warp_max(m);
+  __shared__ double s_l[8], s_m[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0) {
+    s_l[warp] = loss;
+    s_m[warp] = m;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) {
+      loss += s_l[w];
+      m = fmax(m, s_m[w]);
+    }
+    atomicAdd(out, loss);
+    atomic_max_nonneg(out + 1, m);
+  }
+}
+
+__global__ void k_adjoint_rhs(int N, int R, double* __restrict__ v, double* __restrict__ vmax, double* __restrict__ cg,
+                              int* __restrict__ hist) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  double m = 0.0;
+  if (i < N) {
+    v[i] = -v[i];
+    m = fabs(v[i]);
+  }
+  m = warp_max(m);
+  if ((threadIdx.x & 31) == 0 && m > 0.0) atomic_max_nonneg(vmax, m);
+  if (i < R) cg[(size_t)i * CG_STRIDE + CG_Q] = 0.0;
+  if (i == 0) *hist = 0;
+}
+
 // ---------------------------------------------------------------- launchers
+void launch_force_residual(const DevState& S, const double* F_ref, const int* order, const double* wF, double* g,
+                           double* out, cudaStream_t st) {
+  if (S.N == 0) return;
+  k_force_residual<<<(S.N + 255) / 256, 256, 0, st>>>(S.N, S.F, F_ref, order, S.rep, wF, g, out);
+}
+
+void launch_adjoint_rhs(const DevState& S, double* v, double* vmax, cudaStream_t st) {
+  const int n = std::max(S.N, S.R);
+  k_adjoint_rhs<<<(n + 255) / 256, 256, 0, st>>>(S.N, S.R, v, vmax, S.cg, S.cg_hist);
+}
+
 template <class R, class S>
 static cudaError_t pgrad_launch(const DevState& D, const ParamsT<R>& P, const ctbop_params& P64, const double* wval, const double* wtan,
                                 const double* dir, const double* qdir, double* grad, double* vout,

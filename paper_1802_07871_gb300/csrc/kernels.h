@@ -227,6 +227,14 @@ cudaError_t tune_cov(DevState& S, const PotParams<R>& P, const TypeParams& T, cu
 cudaError_t launch_param_grad(const DevState& S, const ::ctbop_params& P, bool fp32, const double* wval,
                               const double* wtan, const double* dir, const double* qdir, double* grad,
                               double* vout, cudaStream_t st);
+// Force-matching residual: g = 2 w_F (F - F_ref) per atom ([N,3], storage
+// order; F_ref in the caller's, through order when it is not null), out[0] +=
+// sum_r w_F |F - F_ref|^2, out[1] = max |g|.
+void launch_force_residual(const DevState& S, const double* F_ref, const int* order, const double* wF, double* g,
+                           double* out, cudaStream_t st);
+// v = -v and *vmax = max |v|; the charge solver's state for an adjoint solve
+// from zero with no total charge.
+void launch_adjoint_rhs(const DevState& S, double* v, double* vmax, cudaStream_t st);
 // Energy minimisation (csrc/relax.cu): one FIRE state per replica,
 // [R][FI_STRIDE] doubles; FI_P..FI_FMAX2 are the per-iteration sums.
 enum FireSlots {
