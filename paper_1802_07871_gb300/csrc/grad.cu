@@ -352,7 +352,8 @@ __global__ void __launch_bounds__(NT)
           ent_vec(ek, kx, ky, kz, rk);
           const S fck = Mk<S>::f(ek.fc, ek.tfc);
           const S ct = ex * kx + ey * ky + ez * kz, dr = re - rk;
-          const bool taper = ek.fc != R(1);
+          // (by the length: just past R the cutoff rounds to 1 while its second derivative has already jumped)
+          const bool taper = val(rk) >= P.R_[pk];
           S fkR, fkS, dum;
           if (taper) fc_params(rk, P.R_[pk], P.S[pk], dum, fkR, fkS);
 #pragma unroll
