@@ -175,6 +175,17 @@ __device__ inline int wrap_cell(int c, int n) {
 // the largest covalent count, the largest count of the rest (the list needs
 // cap_cov + that) and the largest total.
 //
+// The tests run in FP32 for both policies. An FP64 warp instruction takes 64
+// cycles of a scheduler, and a pair test in FP64 eleven of them; so the FP64
+// policy tests in FP32, with a bound on that test's rounding, and takes the
+// FP64 distance only where some lane's FP32 one lies within the bound of a
+// limit (a few in a million pairs): the rows are those of FP64 tests. The
+// bound: 6 roundings of 2^-24 of the coordinates that enter a component,
+// twice the radius times that for each of three components, doubled.
+//
+// With FP64 and FP32 tests: the lists' share of an MD step of 19,555 atoms 220
+// and 106 us, an evaluation of 64 atoms at new positions 800 and 695 us.
+//
 // BW (warps per block) and BC (stencil cells per batch) only change how the
 // cells are spread over blocks and how the stencil is chunked; every shape
 // writes the same rows (see tune_build).
@@ -187,12 +198,15 @@ __global__ void __launch_bounds__(BW * 32)
             int* __restrict__ ncov, int* __restrict__ nfix, int* __restrict__ nall, int* __restrict__ maxcnt,
             unsigned* __restrict__ err, const int* __restrict__ flag) {
   typedef typename Vec4<R>::T R4;
+  constexpr bool EX = sizeof(R) == 8;   // FP32 tests that may need the FP64 distance
   __shared__ int s_st[BW][BC], s_pre[BW][BC + 1], s_cd[BW][BC];
-  __shared__ R4 s_u[BW][32];
+  __shared__ float4 s_u[BW][32];
+  __shared__ R4 s_ux[EX ? BW : 1][EX ? 32 : 1];   // the same in FP64
   __shared__ int s_i[BW][32];
   __shared__ int s_need[BW][3];
   // candidates that passed the box test, first in first out (up to 63 held)
-  __shared__ R4 s_cu[BW][64];
+  __shared__ float4 s_cu[BW][64];
+  __shared__ R4 s_cx[EX ? BW : 1][EX ? 64 : 1];
   __shared__ int s_cj[BW][64], s_cc[BW][64];
   if (*flag == 0) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -200,10 +214,14 @@ __global__ void __launch_bounds__(BW * 32)
   int need_cov = 0, need_rest = 0, need_tot = 0;   // this lane's maxima over the atoms it owned
   // the largest list radius squared, widened by 1e-4 (relative) so that
   // rounding never drops a candidate the pair test below would keep
-  R r2max = P.rall_list2;
+  float r2max = (float)P.rall_list2;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) r2max = max(r2max, P.rcov_list2[k]);
-  r2max *= R(1.0001);
+  for (int k = 0; k < 4; ++k) r2max = fmaxf(r2max, (float)P.rcov_list2[k]);
+  // (FP64 policy) rounding of an FP32 squared distance near the limits, per
+  // unit of the coordinates' size
+  const float eps = EX ? 48.0f * 5.9604645e-8f * sqrtf(r2max) : 0.0f;
+  r2max *= 1.0001f;
+  const float core2 = (float)P.rcore_list2, all2 = (float)P.rall_list2;
   for (int g = blockIdx.x * BW + warp; g < C; g += gridDim.x * BW) {
     int nci = cell_count[g];
     if (nci == 0) continue;
@@ -211,18 +229,20 @@ __global__ void __launch_bounds__(BW * 32)
     const RepInfo& ri = reps[cell_rep[g]];
     const int loc = g - ri.cell_off;
     const int cx = loc % ri.n[0], cy = (loc / ri.n[0]) % ri.n[1], cz = loc / (ri.n[0] * ri.n[1]);
-    const R hx = (R)ri.hc[0], hy = (R)ri.hc[1], hz = (R)ri.hc[2];
+    const float hx = (float)ri.hc[0], hy = (float)ri.hc[1], hz = (float)ri.hc[2];
     const int sx = 2 * ri.m[0] + 1, sy = 2 * ri.m[1] + 1;
     const int ns = sx * sy * (2 * ri.m[2] + 1);
     for (int ib = 0; ib < nci; ib += 32) {
       const int ni = min(32, nci - ib);
       int my_i = -1, cnt_c = 0, cnt_k = 0, cnt_s = 0;
       // bounding box of this group's atoms (offsets from the cell origin)
-      R lox = R(1e30), loy = R(1e30), loz = R(1e30), hix = R(-1e30), hiy = R(-1e30), hiz = R(-1e30);
+      float lox = 1e30f, loy = 1e30f, loz = 1e30f, hix = -1e30f, hiy = -1e30f, hiz = -1e30f;
       if (lane < ni) {
         my_i = cell_atoms[ci0 + ib + lane];
-        const R4 ui = u[my_i];
+        const R4 ux = u[my_i];
+        const float4 ui = make_float4((float)ux.x, (float)ux.y, (float)ux.z, (float)ux.w);
         s_u[warp][lane] = ui;
+        if (EX) s_ux[EX ? warp : 0][EX ? lane : 0] = ux;
         s_i[warp][lane] = my_i;
         lox = hix = ui.x;
         loy = hiy = ui.y;
@@ -230,49 +250,80 @@ __global__ void __launch_bounds__(BW * 32)
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        lox = min(lox, __shfl_xor_sync(CT_FULL, lox, o));
-        loy = min(loy, __shfl_xor_sync(CT_FULL, loy, o));
-        loz = min(loz, __shfl_xor_sync(CT_FULL, loz, o));
-        hix = max(hix, __shfl_xor_sync(CT_FULL, hix, o));
-        hiy = max(hiy, __shfl_xor_sync(CT_FULL, hiy, o));
-        hiz = max(hiz, __shfl_xor_sync(CT_FULL, hiz, o));
+        lox = fminf(lox, __shfl_xor_sync(CT_FULL, lox, o));
+        loy = fminf(loy, __shfl_xor_sync(CT_FULL, loy, o));
+        loz = fminf(loz, __shfl_xor_sync(CT_FULL, loz, o));
+        hix = fmaxf(hix, __shfl_xor_sync(CT_FULL, hix, o));
+        hiy = fmaxf(hiy, __shfl_xor_sync(CT_FULL, hiy, o));
+        hiz = fmaxf(hiz, __shfl_xor_sync(CT_FULL, hiz, o));
       }
       __syncwarp();
       // Pair tests of the first n staged candidates (one per lane) against
       // every atom of the group, in staging order, which is stencil order:
       // each row receives its entries in the same order as without staging.
+      const float size_i = fmaxf(fmaxf(fmaxf(fabsf(lox), fabsf(hix)), fmaxf(fabsf(loy), fabsf(hiy))),
+                                 fmaxf(fabsf(loz), fabsf(hiz)));
+      auto size_of = [&](const float4& c, float ox, float oy, float oz) {
+        return size_i + fmaxf(fabsf(c.x) + fabsf(ox), fmaxf(fabsf(c.y) + fabsf(oy), fabsf(c.z) + fabsf(oz)));
+      };
       auto pair_tests = [&](int n) {
         const bool valid = lane < n;
         int j = -1, cd = 0;
-        R4 uj;
-        uj.x = uj.y = uj.z = uj.w = R(0);
-        R ox = R(0), oy = R(0), oz = R(0);
+        float4 uj = make_float4(0.f, 0.f, 0.f, 0.f);
+        float ox = 0.f, oy = 0.f, oz = 0.f, tol = 0.f;
         if (valid) {
           uj = s_cu[warp][lane];
           j = s_cj[warp][lane];
           cd = s_cc[warp][lane];
           int dx, dy, dz;
           unpack_code(cd, dx, dy, dz);
-          ox = (R)dx * hx;
-          oy = (R)dy * hy;
-          oz = (R)dz * hz;
+          ox = (float)dx * hx;
+          oy = (float)dy * hy;
+          oz = (float)dz * hz;
+          if (EX) tol = eps * size_of(uj, ox, oy, oz);
         }
         const int tj = (int)uj.w;
         const bool zero_off = cd == pack_code(0, 0, 0);
+        // (FP64 policy) covalent limits with an atom of type 0 and of type 1, rounded
+        const float cov0 = (float)P.rcov_list2[tj], cov1 = (float)P.rcov_list2[2 + tj];
         for (int ii = 0; ii < ni; ++ii) {
-          const R4 ui = s_u[warp][ii];
+          const float4 ui = s_u[warp][ii];
           const int i = s_i[warp][ii];
-          R rx = (uj.x - ui.x) + ox, ry = (uj.y - ui.y) + oy, rz = (uj.z - ui.z) + oz;
-          R r2 = rx * rx + ry * ry + rz * rz;
-          bool self0 = zero_off && j == i;
-          bool in = valid && !self0;
-          bool cov = in && r2 < P.rcov_list2[(int)ui.w * 2 + tj];
-          bool core = in && !cov && r2 < P.rcore_list2;
-          bool shell = in && !cov && !core && r2 < P.rall_list2;
-          unsigned bc = __ballot_sync(CT_FULL, cov), bk = __ballot_sync(CT_FULL, core);
-          unsigned bs = __ballot_sync(CT_FULL, shell);
-          int bcc = __shfl_sync(CT_FULL, cnt_c, ii), bck = __shfl_sync(CT_FULL, cnt_k, ii);
-          int bcs = __shfl_sync(CT_FULL, cnt_s, ii);
+          const float rx = (uj.x - ui.x) + ox, ry = (uj.y - ui.y) + oy, rz = (uj.z - ui.z) + oz;
+          const float r2 = rx * rx + ry * ry + rz * rz;
+          const bool self0 = zero_off && j == i;
+          const bool in = valid && !self0;
+          bool cov, core, shell;
+          if constexpr (EX) {
+            const float c2 = ui.w != 0.f ? cov1 : cov0;
+            bool near = r2 < c2, mid = r2 < core2, far = r2 < all2;
+            const bool amb = in && (fabsf(r2 - c2) <= tol || fabsf(r2 - core2) <= tol || fabsf(r2 - all2) <= tol);
+            if (__any_sync(CT_FULL, amb)) {
+              if (amb) {
+                const R4 xj = s_cx[warp][lane], xi = s_ux[warp][ii];
+                int dx, dy, dz;
+                unpack_code(cd, dx, dy, dz);
+                const R ax = (xj.x - xi.x) + (R)dx * (R)ri.hc[0], ay = (xj.y - xi.y) + (R)dy * (R)ri.hc[1],
+                        az = (xj.z - xi.z) + (R)dz * (R)ri.hc[2];
+                const R a2 = ax * ax + ay * ay + az * az;
+                near = a2 < P.rcov_list2[(int)ui.w * 2 + tj];
+                mid = a2 < P.rcore_list2;
+                far = a2 < P.rall_list2;
+              }
+              __syncwarp();
+            }
+            cov = in && near;
+            core = in && !near && mid;
+            shell = in && !near && !mid && far;
+          } else {
+            cov = in && r2 < P.rcov_list2[(int)ui.w * 2 + tj];
+            core = in && !cov && r2 < core2;
+            shell = in && !cov && !core && r2 < all2;
+          }
+          const unsigned bc = __ballot_sync(CT_FULL, cov), bk = __ballot_sync(CT_FULL, core);
+          const unsigned bs = __ballot_sync(CT_FULL, shell);
+          const int bcc = __shfl_sync(CT_FULL, cnt_c, ii), bck = __shfl_sync(CT_FULL, cnt_k, ii);
+          const int bcs = __shfl_sync(CT_FULL, cnt_s, ii);
           if (cov) {
             int pos = bcc + __popc(bc & lt);
             if (pos < cap_cov) lst[(size_t)i * cap_all + pos] = make_int2(j, cd);
@@ -339,7 +390,8 @@ __global__ void __launch_bounds__(BW * 32)
           const int t = t0 + lane;
           bool keep = false;
           int j = -1, cd = 0;
-          R4 uj;
+          R4 ux;
+          float4 uj;
           if (t < T) {
             int lo = 0, hi = nb;   // largest k with s_pre[k] <= t
             while (hi - lo > 1) {
@@ -348,21 +400,25 @@ __global__ void __launch_bounds__(BW * 32)
             }
             j = cell_atoms[s_st[warp][lo] + (t - s_pre[warp][lo])];
             cd = s_cd[warp][lo];
-            uj = u[j];
+            ux = u[j];
+            uj = make_float4((float)ux.x, (float)ux.y, (float)ux.z, (float)ux.w);
             int dx, dy, dz;
             unpack_code(cd, dx, dy, dz);
             // distance from the candidate's image to the group's box: past
             // the list radius, no atom of the group can take it
-            const R px = uj.x + (R)dx * hx, py = uj.y + (R)dy * hy, pz = uj.z + (R)dz * hz;
-            const R bx = max(max(lox - px, px - hix), R(0));
-            const R by = max(max(loy - py, py - hiy), R(0));
-            const R bz = max(max(loz - pz, pz - hiz), R(0));
-            keep = bx * bx + by * by + bz * bz <= r2max;
+            const float ox = (float)dx * hx, oy = (float)dy * hy, oz = (float)dz * hz;
+            const float px = uj.x + ox, py = uj.y + oy, pz = uj.z + oz;
+            const float bx = fmaxf(fmaxf(lox - px, px - hix), 0.f);
+            const float by = fmaxf(fmaxf(loy - py, py - hiy), 0.f);
+            const float bz = fmaxf(fmaxf(loz - pz, pz - hiz), 0.f);
+            const float lim = EX ? r2max + eps * size_of(uj, ox, oy, oz) : r2max;
+            keep = bx * bx + by * by + bz * bz <= lim;
           }
           const unsigned bk = __ballot_sync(CT_FULL, keep);
           if (keep) {
             const int pos = nst + __popc(bk & lt);
             s_cu[warp][pos] = uj;
+            if (EX) s_cx[EX ? warp : 0][EX ? pos : 0] = ux;
             s_cj[warp][pos] = j;
             s_cc[warp][pos] = cd;
           }
@@ -372,7 +428,8 @@ __global__ void __launch_bounds__(BW * 32)
             pair_tests(32);
             // move the rest (fewer than 32) to the front
             if (lane < nst - 32) {
-              const R4 a = s_cu[warp][32 + lane];
+              const float4 a = s_cu[warp][32 + lane];
+              if (EX) s_cx[EX ? warp : 0][EX ? lane : 0] = s_cx[EX ? warp : 0][EX ? 32 + lane : 0];
               const int b = s_cj[warp][32 + lane], c = s_cc[warp][32 + lane];
               s_cu[warp][lane] = a;
               s_cj[warp][lane] = b;
