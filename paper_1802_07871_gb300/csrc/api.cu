@@ -463,6 +463,8 @@ static int alloc_lists(ctbop_system* s, int cap_cov, int cap_all) {
   S.bo = bo;
   S.gslot = gs;
   S.M = M;
+  S.kd = nullptr;
+  if (!s->mixed && stored_kernel(S)) CK(dalloc(s->list_buf, &S.kd, ncol));
   if (cap_cov > 512) return fail(s, CTBOP_ERR_NEIGH_OVERFLOW, "covalent entries per atom beyond 512");
   CK(s->mixed ? setup_pot<float>(cap_cov, &S.cov_lanes_ok) : setup_pot<double>(cap_cov, &S.cov_lanes_ok));
   if (!(S.cov_lanes_ok & (S.cov_lanes == 4 ? 1 : S.cov_lanes == 8 ? 2 : 4))) {
@@ -532,7 +534,7 @@ static void enqueue_back(ctbop_system* s, const PotParams<Rr>& P, cudaStream_t s
                          bool solve) {
   DevState& S = s->S;
   if (solve && S.solver == SOLVE_LAUNCHES) launch_cg_end<Rr>(S, st);
-  launch_forces<Rr>(S, P, s->T, md ? 1 : 0, 0.5 * dt, st, !md);
+  launch_forces<Rr>(S, P, s->T, md ? 1 : 0, 0.5 * dt, st, !md, solve);
   if (md && s->nvt) launch_nh_end(S, dt, st);
 }
 
@@ -777,7 +779,7 @@ static int refresh_virial(ctbop_system* s, const PotParams<Rr>& P) {
   DevState& S = s->S;
   launch_cov_force<Rr>(S, P, s->T, s->stream);
   CK(cudaMemsetAsync(S.rep_acc, 0, sizeof(double) * (size_t)s->R * RA_STRIDE, s->stream));
-  launch_coul_gather<Rr>(S, P, s->T, 0, 0.0, s->stream, true);
+  launch_coul_gather<Rr>(S, P, s->T, 0, 0.0, s->stream, true, true);
   CK(cudaGetLastError());
   s->virial_stale = false;
   return CTBOP_OK;
@@ -844,7 +846,7 @@ static int profile_t(ctbop_system* s, const PotParams<Rr>& P, int64_t n, double 
     if (!rc && !whole) rc = timed(7, 2, [&] { launch_cg_end<Rr>(S, st); });
     if (!rc) rc = timed(8, sizeof(Rr) == 4 ? 3 : 1, [&] { launch_cov_force<Rr>(S, P, s->T, st); });
     if (!rc) rc = timed(9, s->nvt ? 2 : 1, [&] {
-      launch_coul_gather<Rr>(S, P, s->T, 1, 0.5 * dt, st, false);
+      launch_coul_gather<Rr>(S, P, s->T, 1, 0.5 * dt, st, false, true);
       if (s->nvt) launch_nh_end(S, dt, st);
     });
     if (!rc) {

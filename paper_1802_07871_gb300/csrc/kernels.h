@@ -116,6 +116,7 @@ struct DevState {
   void* gslot = nullptr;        // Real4[N*cap_cov]
   int2* Mf = nullptr;           // FP64 policy, whole-solve kernel: [cap_all*ld] FP32 (j, coefficient) pairs of M
   void* M = nullptr;            // [cap_all*ld] charge matrix: FP32 (j, coefficient) int2 pairs, or FP64 coefficients
+  double2* kd = nullptr;        // [cap_all*ld] FP64, several lanes per atom: k(r), K'(r)/(r ke) of the entries
   void *Dg = nullptr, *dinv = nullptr;   // Real[N]: Hessian diagonal without self-images, Jacobi inverse
   // CG: the iterate is q itself (FP64); the rest in the working precision
   double *cqh1 = nullptr, *cqh2 = nullptr;  // q of the previous two solves
@@ -181,6 +182,8 @@ template <class R> void launch_cg_end(const DevState& S, cudaStream_t st);
 template <class R>
 cudaError_t launch_cg_solve(const DevState& S, const TypeParams& T, double tol, int max_iter, const double* rhs,
                             cudaStream_t st);
+// Whether the FP64 assembly keeps S.kd for this many atoms.
+bool stored_kernel(const DevState& S);
 // Picks S.solver for the current layout (off: atom offsets, host) and list capacities.
 template <class R> cudaError_t plan_cg_solve(DevState& S, const int64_t* off);
 template <class R> void launch_cg_mv(const DevState& S, cudaStream_t st);
@@ -189,11 +192,12 @@ template <class R> void launch_cg_up(const DevState& S, const SolveCfg& cfg, cud
 template <class R> void launch_cov_force(const DevState& S, const PotParams<R>& P, const TypeParams& T,
                                          cudaStream_t st);
 // virial: accumulate the virial (an evaluation) or not (an MD step: the
-// library recomputes it when it is read after steps)
+// library recomputes it when it is read after steps); assembled: the matrix,
+// and in FP64 S.kd with it, was assembled at these positions
 template <class R> void launch_coul_gather(const DevState& S, const PotParams<R>& P, const TypeParams& T,
-                                           int kick, double half_dt, cudaStream_t st, bool virial);
+                                           int kick, double half_dt, cudaStream_t st, bool virial, bool assembled);
 template <class R> void launch_forces(const DevState& S, const PotParams<R>& P, const TypeParams& T,
-                                      int kick, double half_dt, cudaStream_t st, bool virial);
+                                      int kick, double half_dt, cudaStream_t st, bool virial, bool assembled);
 template <class R> void launch_kick_drift(const DevState& S, const TypeParams& T, double dt, double half_skin2,
                                           cudaStream_t st);
 void launch_zero_acc(const DevState& S, cudaStream_t st);

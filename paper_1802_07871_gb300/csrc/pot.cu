@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(LG_T)
                  const int* __restrict__ ncov, const int* __restrict__ nfix, const int* __restrict__ nall,
                  const int* __restrict__ rev, const typename Vec4<R>::T* __restrict__ bo, PotParams<R> P,
                  TypeParams T, void* __restrict__ M, R* __restrict__ Dg, R* __restrict__ dinv,
-                 int* __restrict__ nmat) {
+                 int* __restrict__ nmat, double2* __restrict__ kd) {
   using R4 = typename Vec4<R>::T;
   constexpr int AW = 32 / G;   // atoms per warp
   const int lane = threadIdx.x & 31, a = lane % AW, l = lane / AW;
@@ -545,6 +545,19 @@ __global__ void __launch_bounds__(LG_T)
   const R gs_i0 = P.gshield3[ti * 2], gs_i1 = P.gshield3[ti * 2 + 1];
   const int2* pl = nl + i;
   R wsum = R(0), selfm = R(0);
+  // K(r); in FP64 with k and K'/(r ke) kept at the entry's place for the
+  // charge-force gather (kd), which would compute them again
+  auto charge_kernel = [&](R r2, R wj, size_t off) {
+    const R gs = wj != R(0) ? gs_i1 : gs_i0;
+    if constexpr (sizeof(R) == 8) {
+      R k, d;
+      coul_kd_r2<R>(r2, gs, P.inv_rcoul, P.rcoul2, k, d);
+      kd[off] = make_double2(k, d);
+      return P.ke * k;
+    } else {
+      return coul_K_r2<R>(r2, gs, P.inv_rcoul, P.rcoul2, P.ke);
+    }
+  };
   // covalent entries: K minus twice the bond-order coupling w
   for (int e = l; e < nc; e += G) {
     const int2 jcd = __ldg(pl + (size_t)e * ld);
@@ -554,7 +567,7 @@ __global__ void __launch_bounds__(LG_T)
     rel_vec<R>(ui, uj, jcd.y, hx, hy, hz, rx, ry, rz);
     const R r2 = rx * rx + ry * ry + rz * rz;
     const int pb = ti * 2 + (int)uj.w;
-    R m = coul_K_r2<R>(r2, P.gshield3[pb], P.inv_rcoul, P.rcoul2, P.ke);
+    R m = charge_kernel(r2, uj.w, (size_t)e * ld + i);
     const R r = ct_sqrt<R>(r2);
     if (r < P.Sout[pb]) {
       R fc, dfc;
@@ -569,11 +582,10 @@ __global__ void __launch_bounds__(LG_T)
     if (j == i) selfm += m;
     mat_store(M, (size_t)e * ld + i, j, m);
   }
-  auto kernel = [&](const R4& uj, int cd) {
+  auto kernel = [&](const R4& uj, int cd, size_t off) {
     R rx, ry, rz;
     rel_vec<R>(ui, uj, cd, hx, hy, hz, rx, ry, rz);
-    const R r2 = rx * rx + ry * ry + rz * rz;
-    return coul_K_r2<R>(r2, uj.w != R(0) ? gs_i1 : gs_i0, P.inv_rcoul, P.rcoul2, P.ke);
+    return charge_kernel(rx * rx + ry * ry + rz * rz, uj.w, off);
   };
   // core entries, and in FP64 the shell too: stored at their list row
   const int n1 = sizeof(R) == 8 ? na : nf;
@@ -589,7 +601,7 @@ __global__ void __launch_bounds__(LG_T)
     for (int k = 0; k < LG_B; ++k) {
       const int e = e0 + k * G;
       if (e < n1) {
-        const R m = kernel(uj[k], jc[k].y);
+        const R m = kernel(uj[k], jc[k].y, (size_t)e * ld + i);
         if (jc[k].x == i) selfm += m;
         mat_store(M, (size_t)e * ld + i, jc[k].x, m);
       }
@@ -605,7 +617,7 @@ __global__ void __launch_bounds__(LG_T)
       if (e < na) {
         const int2 jc = __ldg(pl + (size_t)e * ld);
         j = jc.x;
-        m = kernel(u[j], jc.y);
+        m = kernel(u[j], jc.y, (size_t)e * ld + i);
       }
       const unsigned kept = __ballot_sync(CT_FULL, m != R(0)) & mine;
       if (m != R(0)) {
@@ -999,7 +1011,14 @@ __global__ void __launch_bounds__(256, gather_min_blocks<PB, VIR>())
 // are dealt to the lanes, their sums joined by shuffles (the energies with
 // their compensation), and one warp of the block then takes the block's atoms
 // through the FP64 epilogue with full lanes.
-template <class R, int G, bool VIR>
+// ST (FP64): k and K'/(r ke) come from the assembly at these positions
+// (S.kd, 16 bytes per entry each way). Both passes are bound by the FP64
+// pipe, and the kernel's roots and polynomials are two thirds of an entry's
+// FP64 instructions: 19,555 atoms 525 -> 182 us here against 421 -> 526 there;
+// 512 atoms 46 -> 27 against 37 -> 45. FP32 computes them again (its
+// instructions cost less than the bytes), and so does an evaluation at fixed
+// charges, which assembles no matrix.
+template <class R, int G, bool VIR, bool ST>
 __global__ void __launch_bounds__(LG_T)
     k_coul_gather_g(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ u,
                     const int* __restrict__ rep, const RepInfo* __restrict__ reps, const int2* __restrict__ nl,
@@ -1008,7 +1027,7 @@ __global__ void __launch_bounds__(LG_T)
                     const R* __restrict__ qr, PotParams<R> P, TypeParams T, int kick, double half_dt,
                     const uint8_t* __restrict__ frozen, double* __restrict__ F, double* __restrict__ v,
                     double* __restrict__ e_atom, double* __restrict__ rep_acc, unsigned* __restrict__ err,
-                    const double* __restrict__ nh) {
+                    const double* __restrict__ nh, const double2* __restrict__ kd) {
   using R4 = typename Vec4<R>::T;
   constexpr int AW = 32 / G, AB = LG_T / 32 * AW;   // atoms per warp, per block
   constexpr int NS = VIR ? 14 : 5;
@@ -1029,10 +1048,15 @@ __global__ void __launch_bounds__(LG_T)
     const int2* pl = nl + i;
     const R gs_i0 = P.gshield3[ti * 2], gs_i1 = P.gshield3[ti * 2 + 1];
     // charges: qj K and qj K'/r are summed, (ke / 2) qi and ke qi applied once per lane
-    auto add = [&](R rx, R ry, R rz, R wj, R qj, R& en) {
-      const R r2 = rx * rx + ry * ry + rz * rz;
+    auto add = [&](R rx, R ry, R rz, R wj, R qj, double2 st, R& en) {
       R K, c;
-      coul_kd_r2<R>(r2, wj != R(0) ? gs_i1 : gs_i0, P.inv_rcoul, P.rcoul2, K, c);
+      if constexpr (ST) {
+        K = (R)st.x;
+        c = (R)st.y;
+      } else {
+        const R r2 = rx * rx + ry * ry + rz * rz;
+        coul_kd_r2<R>(r2, wj != R(0) ? gs_i1 : gs_i0, P.inv_rcoul, P.rcoul2, K, c);
+      }
       c *= qj;
       // (explicit: the variants with and without the virial round alike)
       s[0] = fma(c, rx, s[0]); s[1] = fma(c, ry, s[1]); s[2] = fma(c, rz, s[2]);
@@ -1048,6 +1072,7 @@ __global__ void __launch_bounds__(LG_T)
       int2 jc[LG_B];
       R4 uj[LG_B];
       R qj[LG_B], en[LG_B];
+      double2 st[LG_B];
 #pragma unroll
       for (int k = 0; k < LG_B; ++k)
         jc[k] = e0 + k * G < na ? __ldg(pl + (size_t)(e0 + k * G) * ld) : make_int2(i, pack_code(0, 0, 0));
@@ -1055,6 +1080,8 @@ __global__ void __launch_bounds__(LG_T)
       for (int k = 0; k < LG_B; ++k) {
         uj[k] = u[jc[k].x];
         qj[k] = qr[jc[k].x];
+        st[k] = make_double2(0.0, 0.0);
+        if (ST) st[k] = __ldg(kd + (e0 + k * G < na ? (size_t)(e0 + k * G) * ld : 0) + i);   // (past the row's end: not used)
       }
 #pragma unroll
       for (int k = 0; k < LG_B; ++k) {
@@ -1062,7 +1089,7 @@ __global__ void __launch_bounds__(LG_T)
         if (e0 + k * G < na) {
           R rx, ry, rz;
           rel_vec<R>(ui, uj[k], jc[k].y, hx, hy, hz, rx, ry, rz);
-          add(rx, ry, rz, uj[k].w, qj[k], en[k]);
+          add(rx, ry, rz, uj[k].w, qj[k], st[k], en[k]);
         }
       }
       if (sizeof(R) == 4) {
@@ -1267,6 +1294,8 @@ static int row_lanes(const DevState& S) {
   return S.N <= S.nsm * (sizeof(R) == 4 ? 32 : 64) ? 32 : S.N <= full ? 8 : 1;
 }
 
+bool stored_kernel(const DevState& S) { return row_lanes<double>(S) > 1; }
+
 template <class R>
 void launch_assemble(const DevState& S, const PotParams<R>& P, const TypeParams& T, cudaStream_t st) {
   if (S.N == 0) return;
@@ -1274,8 +1303,8 @@ void launch_assemble(const DevState& S, const PotParams<R>& P, const TypeParams&
   S.N, S.cap_cov, S.ld, (const typename Vec4<R>::T*)S.u, S.rep, S.reps, S.nl, S.ncov, S.nfix, S.nall, S.rev, \
       (const typename Vec4<R>::T*)S.bo, P, T, S.M, (R*)S.Dg, (R*)S.dinv, S.nmat
   const int g = (S.N + 255) / 256, lanes = row_lanes<R>(S), per = LG_T / lanes;
-  if (lanes == 32) k_assemble_g<R, 32><<<(S.N + per - 1) / per, LG_T, 0, st>>>(ASM_ARGS);
-  else if (lanes == 8) k_assemble_g<R, 8><<<(S.N + per - 1) / per, LG_T, 0, st>>>(ASM_ARGS);
+  if (lanes == 32) k_assemble_g<R, 32><<<(S.N + per - 1) / per, LG_T, 0, st>>>(ASM_ARGS, S.kd);
+  else if (lanes == 8) k_assemble_g<R, 8><<<(S.N + per - 1) / per, LG_T, 0, st>>>(ASM_ARGS, S.kd);
   else if (S.asm_batch == 4) k_assemble<R, 4><<<g, 256, 0, st>>>(ASM_ARGS);
   else if (S.asm_batch == 16) k_assemble<R, 16><<<g, 256, 0, st>>>(ASM_ARGS);
   else k_assemble<R, 8><<<g, 256, 0, st>>>(ASM_ARGS);
@@ -1315,10 +1344,10 @@ void launch_cov_force(const DevState& S, const PotParams<R>& P, const TypeParams
 
 template <class R>
 void launch_coul_gather(const DevState& S, const PotParams<R>& P, const TypeParams& T, int kick, double half_dt,
-                        cudaStream_t st, bool virial) {
+                        cudaStream_t st, bool virial, bool assembled) {
   if (S.N == 0) return;
   const int lanes = row_lanes<R>(S);
-  auto go = [&](auto kernel) {
+  auto go = [&](auto kernel, auto... more) {
     int occ = 0, grid = 0;
     if (lanes > 1) {
       grid = (S.N + LG_T / lanes - 1) / (LG_T / lanes);
@@ -1330,12 +1359,20 @@ void launch_coul_gather(const DevState& S, const PotParams<R>& P, const TypePara
     kernel<<<grid, 256, 0, st>>>(
         S.N, S.cap_cov, S.ld, (const typename Vec4<R>::T*)S.u, S.rep, S.reps, S.nl,
         S.ncov, S.nall, S.rev, (const typename Vec4<R>::T*)S.gslot, (const R*)S.qr, P, T, kick, half_dt,
-        S.frozen, S.F, S.v, S.e_atom, S.rep_acc, S.err, S.nh);
+        S.frozen, S.F, S.v, S.e_atom, S.rep_acc, S.err, S.nh, more...);
   };
-  if (lanes == 32) {
-    if (virial) go(k_coul_gather_g<R, 32, true>); else go(k_coul_gather_g<R, 32, false>);
+  const double2* kd = S.kd;
+  if (sizeof(R) == 8 && lanes > 1 && assembled) {   // (ST = false only with sizeof(R) == 4: never launched there)
+    constexpr bool ST = sizeof(R) == 8;
+    if (lanes == 32) {
+      if (virial) go(k_coul_gather_g<R, 32, true, ST>, kd); else go(k_coul_gather_g<R, 32, false, ST>, kd);
+    } else {
+      if (virial) go(k_coul_gather_g<R, 8, true, ST>, kd); else go(k_coul_gather_g<R, 8, false, ST>, kd);
+    }
+  } else if (lanes == 32) {
+    if (virial) go(k_coul_gather_g<R, 32, true, false>, kd); else go(k_coul_gather_g<R, 32, false, false>, kd);
   } else if (lanes == 8) {
-    if (virial) go(k_coul_gather_g<R, 8, true>); else go(k_coul_gather_g<R, 8, false>);
+    if (virial) go(k_coul_gather_g<R, 8, true, false>, kd); else go(k_coul_gather_g<R, 8, false, false>, kd);
   } else if (virial) {
     if (S.gather_batch == 4) go(k_coul_gather<R, 4, true>);
     else if (S.gather_batch == 6) go(k_coul_gather<R, 6, true>);
@@ -1349,9 +1386,9 @@ void launch_coul_gather(const DevState& S, const PotParams<R>& P, const TypePara
 
 template <class R>
 void launch_forces(const DevState& S, const PotParams<R>& P, const TypeParams& T, int kick, double half_dt,
-                   cudaStream_t st, bool virial) {
+                   cudaStream_t st, bool virial, bool assembled) {
   launch_cov_force<R>(S, P, T, st);
-  launch_coul_gather<R>(S, P, T, kick, half_dt, st, virial);
+  launch_coul_gather<R>(S, P, T, kick, half_dt, st, virial, assembled);
 }
 
 template <class R, int G>
@@ -1533,7 +1570,7 @@ cudaError_t tune_cov(DevState& S, const PotParams<R>& P, const TypeParams& T, cu
     launch_bond<R>(S, P, st);
     launch_cov_force<R>(S, P, T, st);
     cudaMemsetAsync(S.rep_acc, 0, sizeof(double) * (size_t)S.R * RA_STRIDE, st);
-    launch_coul_gather<R>(S, P, T, 0, 0.0, st, true);
+    launch_coul_gather<R>(S, P, T, 0, 0.0, st, true, false);
   }
   for (int k = 0; k < 3; ++k) cudaEventDestroy(ev[k]);
   return e == cudaSuccess ? cudaGetLastError() : e;
@@ -1568,7 +1605,7 @@ cudaError_t tune_gather(DevState& S, const PotParams<R>& P, const TypeParams& T,
       cudaMemsetAsync(S.rep_acc, 0, acc_bytes, st);
       launch_cov_force<R>(S, P, T, st);
       cudaEventRecord(e0, st);
-      launch_coul_gather<R>(S, P, T, 0, 0.0, st, false);   // the variant MD steps run
+      launch_coul_gather<R>(S, P, T, 0, 0.0, st, false, false);   // the variant MD steps run
       cudaEventRecord(e1, st);
       e = cudaEventSynchronize(e1);
       float ms = 0.0f;
@@ -1586,7 +1623,7 @@ cudaError_t tune_gather(DevState& S, const PotParams<R>& P, const TypeParams& T,
   if (e == cudaSuccess) {
     cudaMemsetAsync(S.rep_acc, 0, acc_bytes, st);
     launch_cov_force<R>(S, P, T, st);
-    launch_coul_gather<R>(S, P, T, 0, 0.0, st, true);
+    launch_coul_gather<R>(S, P, T, 0, 0.0, st, true, false);
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -1601,12 +1638,12 @@ template void launch_assemble<double>(const DevState&, const PotParams<double>&,
 template void launch_cov_force<float>(const DevState&, const PotParams<float>&, const TypeParams&, cudaStream_t);
 template void launch_cov_force<double>(const DevState&, const PotParams<double>&, const TypeParams&, cudaStream_t);
 template void launch_coul_gather<float>(const DevState&, const PotParams<float>&, const TypeParams&, int, double,
-                                        cudaStream_t, bool);
+                                        cudaStream_t, bool, bool);
 template void launch_coul_gather<double>(const DevState&, const PotParams<double>&, const TypeParams&, int, double,
-                                         cudaStream_t, bool);
+                                         cudaStream_t, bool, bool);
 template void launch_forces<float>(const DevState&, const PotParams<float>&, const TypeParams&, int, double,
-                                   cudaStream_t, bool);
+                                   cudaStream_t, bool, bool);
 template void launch_forces<double>(const DevState&, const PotParams<double>&, const TypeParams&, int, double,
-                                    cudaStream_t, bool);
+                                    cudaStream_t, bool, bool);
 
 }  // namespace ct
