@@ -504,18 +504,21 @@ __global__ void __launch_bounds__(256)
 // the lanes, a shell entry's place is its rank among the kept ones (ballots),
 // so the matrix has the same entries in the same places. FP64 is bound by its
 // pipe (64 cycles per warp instruction and scheduler): at 512 atoms a thread
-// per atom keeps 2 of 152 SMs busy (1,019 us; 21 with 32 lanes per atom).
-// threads per block: the rows are long and of one length, so the size sets
-// how evenly blocks fall on the SMs (FP64, 256 -> 128 threads: 512 atoms,
+// per atom keeps 2 of 152 SMs busy (1,019 us; 27 with 32 lanes per atom, the
+// derivative for the gather included).
+//
+// Threads per block: the rows are long and of one length, so the size sets
+// how evenly blocks fall on the SMs. 256 -> 128 threads: FP64, 512 atoms,
 // assembly 44 -> 27 and gather 25 -> 18 us; 19,555 atoms 526 -> 490 and
-// 182 -> 175; 64 threads the same within the spread)
-template <class R> constexpr int lg_t = sizeof(R) == 8 ? 128 : 256;
+// 182 -> 175; mixed, 158,391 atoms, gather 162 -> 153 us, assembly the same.
+// 64 threads are no better.
+#define LG_T 128
 #define LG_B 4           // entries in flight per lane
-#define LG_FULL32 1300   // atoms per SM up to which FP32 takes 8 lanes per atom (at 158,391 atoms 172 + 161 us
+#define LG_FULL32 1300   // atoms per SM up to which FP32 takes 8 lanes per atom (at 158,391 atoms 173 + 153 us
                          // against 190 + 205; at 1,005,466 atoms 2,410 + 1,183 against 938 + 970)
 #define LG_FULL64 2000   // the same for FP64 (its rows are bound by the FP64 pipe, not by their loads)
 template <class R, int G>
-__global__ void __launch_bounds__(lg_t<R>)
+__global__ void __launch_bounds__(LG_T)
     k_assemble_g(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ u,
                  const int* __restrict__ rep, const RepInfo* __restrict__ reps, const int2* __restrict__ nl,
                  const int* __restrict__ ncov, const int* __restrict__ nfix, const int* __restrict__ nall,
@@ -525,7 +528,7 @@ __global__ void __launch_bounds__(lg_t<R>)
   using R4 = typename Vec4<R>::T;
   constexpr int AW = 32 / G;   // atoms per warp
   const int lane = threadIdx.x & 31, a = lane % AW, l = lane / AW;
-  const int i = (int)((blockIdx.x * lg_t<R> + threadIdx.x) >> 5) * AW + a;
+  const int i = (int)((blockIdx.x * LG_T + threadIdx.x) >> 5) * AW + a;
   const bool in = i < N;
   unsigned mine = 0u;   // the lanes of this atom
 #pragma unroll
@@ -1023,7 +1026,7 @@ __global__ void __launch_bounds__(256, gather_min_blocks<PB, VIR>())
 // instructions cost less than the bytes), and so does an evaluation at fixed
 // charges, which assembles no matrix.
 template <class R, int G, bool VIR, bool ST>
-__global__ void __launch_bounds__(lg_t<R>)
+__global__ void __launch_bounds__(LG_T)
     k_coul_gather_g(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ u,
                     const int* __restrict__ rep, const RepInfo* __restrict__ reps, const int2* __restrict__ nl,
                     const int* __restrict__ ncov, const int* __restrict__ nall,
@@ -1033,11 +1036,11 @@ __global__ void __launch_bounds__(lg_t<R>)
                     double* __restrict__ e_atom, double* __restrict__ rep_acc, unsigned* __restrict__ err,
                     const double* __restrict__ nh, const double2* __restrict__ kd) {
   using R4 = typename Vec4<R>::T;
-  constexpr int AW = 32 / G, AB = lg_t<R> / 32 * AW;   // atoms per warp, per block
+  constexpr int AW = 32 / G, AB = LG_T / 32 * AW;   // atoms per warp, per block
   constexpr int NS = VIR ? 14 : 5;
   __shared__ R s_v[NS][AB];   // force, energy (sum, compensation), virial
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, a = lane % AW, l = lane / AW;
-  const int i = ((int)blockIdx.x * (lg_t<R> / 32) + warp) * AW + a;
+  const int i = ((int)blockIdx.x * (LG_T / 32) + warp) * AW + a;
   R s[NS];
 #pragma unroll
   for (int k = 0; k < NS; ++k) s[k] = R(0);
@@ -1306,9 +1309,9 @@ void launch_assemble(const DevState& S, const PotParams<R>& P, const TypeParams&
 #define ASM_ARGS                                                                                        \
   S.N, S.cap_cov, S.ld, (const typename Vec4<R>::T*)S.u, S.rep, S.reps, S.nl, S.ncov, S.nfix, S.nall, S.rev, \
       (const typename Vec4<R>::T*)S.bo, P, T, S.M, (R*)S.Dg, (R*)S.dinv, S.nmat
-  const int g = (S.N + 255) / 256, lanes = row_lanes<R>(S), per = lg_t<R> / lanes;
-  if (lanes == 32) k_assemble_g<R, 32><<<(S.N + per - 1) / per, lg_t<R>, 0, st>>>(ASM_ARGS, S.kd);
-  else if (lanes == 8) k_assemble_g<R, 8><<<(S.N + per - 1) / per, lg_t<R>, 0, st>>>(ASM_ARGS, S.kd);
+  const int g = (S.N + 255) / 256, lanes = row_lanes<R>(S), per = LG_T / lanes;
+  if (lanes == 32) k_assemble_g<R, 32><<<(S.N + per - 1) / per, LG_T, 0, st>>>(ASM_ARGS, S.kd);
+  else if (lanes == 8) k_assemble_g<R, 8><<<(S.N + per - 1) / per, LG_T, 0, st>>>(ASM_ARGS, S.kd);
   else if (S.asm_batch == 4) k_assemble<R, 4><<<g, 256, 0, st>>>(ASM_ARGS);
   else if (S.asm_batch == 16) k_assemble<R, 16><<<g, 256, 0, st>>>(ASM_ARGS);
   else k_assemble<R, 8><<<g, 256, 0, st>>>(ASM_ARGS);
@@ -1354,13 +1357,13 @@ void launch_coul_gather(const DevState& S, const PotParams<R>& P, const TypePara
   auto go = [&](auto kernel, auto... more) {
     int occ = 0, grid = 0;
     if (lanes > 1) {
-      grid = (S.N + lg_t<R> / lanes - 1) / (lg_t<R> / lanes);
+      grid = (S.N + LG_T / lanes - 1) / (LG_T / lanes);
     } else {
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 256, 0) != cudaSuccess || occ < 1) occ = 1;
       long long tiles = ((long long)S.N + 255) / 256, slots = (long long)S.nsm * occ;
       grid = (int)(tiles < slots ? tiles : slots);
     }
-    kernel<<<grid, lanes > 1 ? lg_t<R> : 256, 0, st>>>(
+    kernel<<<grid, lanes > 1 ? LG_T : 256, 0, st>>>(
         S.N, S.cap_cov, S.ld, (const typename Vec4<R>::T*)S.u, S.rep, S.reps, S.nl,
         S.ncov, S.nall, S.rev, (const typename Vec4<R>::T*)S.gslot, (const R*)S.qr, P, T, kick, half_dt,
         S.frozen, S.F, S.v, S.e_atom, S.rep_acc, S.err, S.nh, more...);
