@@ -324,8 +324,16 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
   __shared__ R s_hi[3][CS_W][32];
   __shared__ float s_lo[sizeof(R) == 4 ? 3 : 1][CS_W][32];   // (compensations: FP32 sums only)
   __shared__ __align__(16) R s_r[CS_W][32];
-  __shared__ double s_abc[2];
-  __shared__ int s_stop;
+  // Words of the scalars, all written by the boss thread alone. A word is read
+  // only after the first __syncthreads past its store, and stored again only
+  // after an exchange that every reader of the old value entered (an exchange
+  // is a barrier of the block too):
+  __shared__ double s_abc[2];   // alpha, beta: stored after the dots' exchange; c, mean: after that of y's sums
+  __shared__ int s_stop;        // max |r - mean| met the goal: stored after the exchange of y's sums
+  __shared__ int s_fell;        // (FP64) the residual fell tenfold: stored after a cycle's first exchange of y's sums
+  __shared__ double s_shift;    // (FP64) the shift with the mean: stored after the CG of a cycle
+  // (s_tot: stored by the exchanges between two of their own barriers, read by
+  // any thread after an exchange and before it enters the next)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // the thread that forms the scalars: of the last warp, which owns no group
   // unless the block has all it can, so its divisions run beside the update
@@ -677,10 +685,14 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
           } else {
             test(s_tot[0], s_tot[1], s_tot[2], s_tot[3], A.tol);
           }
+          if constexpr (sizeof(R) == 8) {
+            s_fell = bound <= 0.1 * last ? 1 : 0;
+            last = bound;
+          }
         }
         __syncthreads();
         conv = s_stop;
-        if (conv || its >= A.max_iter) break;   // (uniform)
+        if (conv || its >= A.max_iter) break;   // (uniform: s_stop stays until the next exchange)
         double dq = 0.0;
         bool go;
         if constexpr (sizeof(R) == 4) {
@@ -691,13 +703,7 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
           if (!go) alive = false;
           break;
         } else {
-          // the boss knows the residual; whether it fell tenfold, for all
-          if (boss) {
-            s_stop = bound <= 0.1 * last ? 1 : 0;
-            last = bound;
-          }
-          __syncthreads();
-          const bool fell = s_stop != 0;
+          const bool fell = s_fell != 0;
           if (fell) {
             go = iterate((float)ri, yf, fmax(0.3 * A.tol, bound * CS_CUT), dq);
           } else {
@@ -720,11 +726,10 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
           // the mean is part of the shift from here on (the boss's, to all)
           if (boss) {
             shift += mean;
-            s_abc[0] = shift;
+            s_shift = shift;
           }
           __syncthreads();
-          shift = s_abc[0];
-          __syncthreads();
+          shift = s_shift;
         }
       }
       if (!alive) break;
