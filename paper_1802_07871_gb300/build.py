@@ -18,6 +18,9 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libctbop.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
+# a function that can end without its return value is an error (the compiler
+# only warns, and its output is shown on failure alone)
+STRICT = ["--diag-error", "940"]
 SOURCES = ["api.cu", "nbr.cu", "pot.cu", "cg.cu", "cgsolve.cu", "md.cu", "noalloc.cu", "grad.cu", "screen.cu", "relax.cu", "rings.cu", "order.cu", "peaks.cu"]
 
 
@@ -29,7 +32,7 @@ def _nvcc() -> str:
 
 
 def _flags(extra=()):
-    return ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2",
+    return ARCH + STRICT + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2",
                    "-I", INCLUDE, "-I", CSRC, *extra]
 
 

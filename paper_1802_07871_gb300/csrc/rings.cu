@@ -316,6 +316,8 @@ __device__ bool ring_search(int a, const RingTable<R>& T, const RingGraph<R>& G,
       dist[depth] = D;
     }
   }
+  __syncwarp();
+  return true;
 }
 
 template <class R>
