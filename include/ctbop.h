@@ -315,7 +315,8 @@ int ctbop_param_grad(ctbop_system* s, const double* w_E, const double* E_ref, co
  * is kept for the next call (its device memory grows with max_atoms).
  * dE: host, n_cand doubles, caller-owned. Errors: INVALID_ARG (an index
  * outside [0, N), null arrays), STATE (no layout, box, types or positions),
- * CG_NOT_CONVERGED (a batch solve), OOM, CUDA. */
+ * CG_NOT_CONVERGED, NONFINITE (the system's state or a batch solve; dE is
+ * written all the same), OOM, CUDA. */
 int ctbop_removal_energies(ctbop_system* s, int64_t n_cand, const int64_t* cand, int64_t max_atoms, double* dE);
 
 /* Energy minimisation (the paper relaxes structures and cools them to 0 K,

@@ -1617,7 +1617,9 @@ int ctbop_energy_noalloc(ctbop_system* s, double* energy) {
 // (s->loo, kept between calls): candidates are grouped by source replica, a
 // chunk holds as many as fit in max_atoms, and a device gather builds each
 // chunk from the current state. The batch's starting charges are the
-// source's (the solver shifts them onto the replica total).
+// source's (the solver shifts them onto the replica total). The error words of
+// the system and of every chunk's solve come back with the energies: a solve
+// that failed or did not converge makes the call fail, after all chunks.
 int ctbop_removal_energies(ctbop_system* s, int64_t n_cand, const int64_t* cand, int64_t max_atoms, double* dE) {
   if (!s) return CTBOP_ERR_INVALID_ARG;
   if (n_cand < 0 || (n_cand > 0 && (!cand || !dE))) return fail(s, CTBOP_ERR_INVALID_ARG, "bad candidate arrays");
@@ -1638,7 +1640,9 @@ int ctbop_removal_energies(ctbop_system* s, int64_t n_cand, const int64_t* cand,
   std::vector<double> E(R);
   std::vector<int> types(N);
   CK(cudaMemcpy2DAsync(E.data(), 8, S.rep_acc + RA_E, RA_STRIDE * 8, 8, R, cudaMemcpyDeviceToHost, s->stream));
+  CK(cudaMemcpyAsync(s->h_int, S.err, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
   CK(sync_copy(s, types.data(), S.type, sizeof(int) * N, cudaMemcpyDeviceToHost));
+  unsigned bits = (unsigned)*s->h_int;
   struct Job { int64_t c; int r; int n; int drop; };
   std::vector<Job> jobs;
   for (int64_t c = 0; c < n_cand; ++c) {
@@ -1742,7 +1746,9 @@ int ctbop_removal_energies(ctbop_system* s, int64_t n_cand, const int64_t* cand,
     std::vector<double> El(C);
     CK(cudaMemcpy2DAsync(El.data(), 8, L->S.rep_acc + RA_E, RA_STRIDE * 8, 8, C, cudaMemcpyDeviceToHost,
                          s->stream));
+    CK(cudaMemcpyAsync(L->h_int, L->S.err, sizeof(unsigned), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
+    bits |= (unsigned)*L->h_int;
     for (size_t k = 0; k < j1 - j0; ++k) {
       const Job& jb = chunk[k];
       dE[jb.c] = El[k] + s->T.E0[types[s->off[jb.r] + jb.drop]] - E[jb.r];
@@ -1750,6 +1756,9 @@ int ctbop_removal_energies(ctbop_system* s, int64_t n_cand, const int64_t* cand,
     j0 = j1;
   }
   CK(cudaStreamSynchronize(s->stream));
+  if (bits & CT_ERR_NONFINITE) return fail(s, CTBOP_ERR_NONFINITE, "removal energies: non-finite energy, force or position");
+  if (bits & CT_ERR_SOLVER) return fail(s, CTBOP_ERR_CUDA, "internal: the charge solve gave up waiting");
+  if (bits & CT_ERR_CG_MAXITER) return fail(s, CTBOP_ERR_CG_NOT_CONVERGED, "removal energies: charge CG reached max_iter");
   return CTBOP_OK;
 }
 
