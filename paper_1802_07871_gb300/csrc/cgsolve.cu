@@ -854,18 +854,11 @@ cudaError_t plan_cg_solve(DevState& S, const int64_t* off) {
   // stored entries per atom: the list's capacity less its headroom and skin
   const double row = 0.65 * S.cap_all * (sizeof(R) == 4 ? 8.0 : 12.0);
   const double l2 = 100e6;
-  int dev = 0, lim = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e != cudaSuccess) return e;
+  size_t most_smem = 0;
+  cudaError_t e = cudaSuccess;
   const bool many = S.R > 1;
   if (ng <= CS_CLMAX * CS_W && (many ? (double)S.N * row <= 3.5 * l2 : maxn <= CS_CL_ONE)) {
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, k_cg_solve<R, true>);
-    if (e != cudaSuccess) return e;
-    // (always the same limit: the attribute is the function's, shared by every system)
-    e = cudaFuncSetAttribute(k_cg_solve<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             lim - (int)fa.sharedSizeBytes);
+    e = allow_dynamic_smem((const void*)k_cg_solve<R, true>, &most_smem);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_cg_solve<R, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
@@ -890,7 +883,7 @@ cudaError_t plan_cg_solve(DevState& S, const int64_t* off) {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int fit = 0;
-    if (cfg.dynamicSmemBytes <= (size_t)(lim - (int)fa.sharedSizeBytes) &&
+    if (cfg.dynamicSmemBytes <= most_smem &&
         cudaOccupancyMaxActiveClusters(&fit, k_cg_solve<R, true>, &cfg) == cudaSuccess && fit > 0) {
       S.solver = SOLVE_CLUSTER;
       S.solve_blocks = size;
@@ -905,14 +898,10 @@ cudaError_t plan_cg_solve(DevState& S, const int64_t* off) {
     // takes off the passes
     const int most = std::min(S.nsm, SOLVE_MAX_BLOCKS), per = (ng + most - 1) / most;
     const size_t smem = solve_smem<R, false>(per, 0, S.precond);
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, k_cg_solve<R, false>);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_cg_solve<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               lim - (int)fa.sharedSizeBytes);
+    e = allow_dynamic_smem((const void*)k_cg_solve<R, false>, &most_smem);
     if (e != cudaSuccess) return e;
     int occ = 0;
-    if (per <= CS_W && smem <= (size_t)(lim - (int)fa.sharedSizeBytes) &&
+    if (per <= CS_W && smem <= most_smem &&
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg_solve<R, false>, CS_T, smem) == cudaSuccess && occ > 0) {
       S.solver = SOLVE_GRID;
       S.solve_blocks = (ng + per - 1) / per;

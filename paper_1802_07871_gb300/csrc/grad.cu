@@ -714,16 +714,11 @@ static cudaError_t pgrad_launch(const DevState& D, const ParamsT<R>& P, const ct
   auto cov = [&](auto kernel, int threads, bool& fits) -> cudaError_t {
     const int apb = threads / PgLanes<R>::v;
     const size_t sm = (size_t)apb * D.cap_cov * (sizeof(Ent<R>) + 3 * sizeof(int));
-    cudaFuncAttributes fa;
-    int dev = 0, lim = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+    size_t most = 0;
+    cudaError_t e = allow_dynamic_smem((const void*)kernel, &most);
     if (e != cudaSuccess) return e;
-    fits = sm + fa.sharedSizeBytes <= (size_t)lim;
-    if (!fits && threads > 32) return cudaSuccess;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
+    fits = sm <= most;
+    if (!fits) return threads > 32 ? cudaSuccess : cudaErrorInvalidValue;
     kernel<<<(D.N + apb - 1) / apb, threads, sm, st>>>(D.N, D.cap_cov, D.ld, (const R4*)D.u, D.rep, D.reps, D.nl,
                                                           D.ncov, D.q, qdir, wval, wtan, dir, P, K, grad, vout);
     return cudaGetLastError();

@@ -157,6 +157,21 @@ struct DevState {
   void* stage = nullptr;        // [N * 24 bytes] staging for per-atom inputs and outputs in the caller's order
 };
 
+// Allows a kernel as much dynamic shared memory as the device has beside its
+// static one, *most. Always the same limit, because the attribute is the
+// function's and every system of the process shares it: a limit of one
+// system's need would refuse the launches of another that needs more.
+inline cudaError_t allow_dynamic_smem(const void* kernel, size_t* most) {
+  cudaFuncAttributes fa;
+  int dev = 0, lim = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+  if (e != cudaSuccess) return e;
+  *most = (size_t)lim - fa.sharedSizeBytes;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*most);
+}
+
 // The forms of the charge solve: two launches per iteration (cg.cu), or one
 // kernel per solve with a thread-block cluster per replica or all blocks on
 // one replica (cgsolve.cu).

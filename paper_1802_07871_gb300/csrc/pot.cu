@@ -1399,42 +1399,35 @@ void launch_forces(const DevState& S, const PotParams<R>& P, const TypeParams& T
 }
 
 template <class R, int G>
-static cudaError_t setup_pot_g(int cap_cov) {
-  cudaError_t e = cudaFuncSetAttribute(k_bond<R, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)bond_smem<R>(cap_cov, G));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_cov_force<R, R, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)force_smem<R>(cap_cov, G));
+static cudaError_t setup_pot_g(int cap_cov, bool& fits) {
+  fits = true;
+  auto allow = [&](auto kernel, size_t need) {
+    size_t most = 0;
+    cudaError_t e = allow_dynamic_smem((const void*)kernel, &most);
+    fits = fits && need <= most;
+    return e;
+  };
+  cudaError_t e = allow(k_bond<R, G>, bond_smem<R>(cap_cov, G));
+  if (e == cudaSuccess) e = allow(k_cov_force<R, R, G>, force_smem<R>(cap_cov, G));
   if (e != cudaSuccess || sizeof(R) == 8) return e;
   // the FP32 path's FP64 pass over queued atoms
-  e = cudaFuncSetAttribute(k_bond<double, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)bond_smem<double>(cap_cov, G));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_cov_force<double, float, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)force_smem<double>(cap_cov, G));
+  e = allow(k_bond<double, G>, bond_smem<double>(cap_cov, G));
+  if (e == cudaSuccess) e = allow(k_cov_force<double, float, G>, force_smem<double>(cap_cov, G));
+  return e;
 }
 
-// Allow the dynamic shared memory the covalent kernels need for cap_cov
-// entries per atom (call before launching or capturing them), at each lane
-// count whose blocks fit the per-block limit: fewer lanes per atom stage
-// more atoms per block. *lanes_ok gets a bit per usable count (1: 4 lanes,
-// 2: 8, 4: 16); 16 lanes must fit.
+// Allow the covalent kernels dynamic shared memory (call before launching or
+// capturing them), and at which lane counts the blocks of cap_cov entries per
+// atom fit: fewer lanes per atom stage more atoms per block. *lanes_ok gets a
+// bit per usable count (1: 4 lanes, 2: 8, 4: 16); 16 lanes must fit.
 template <class R>
 cudaError_t setup_pot(int cap_cov, int* lanes_ok) {
-  int dev = 0, lim = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e != cudaSuccess) return e;
-  auto fits = [&](int G) {
-    size_t need = std::max(force_smem<R>(cap_cov, G), bond_smem<R>(cap_cov, G));
-    if (sizeof(R) == 4) need = std::max(need, force_smem<double>(cap_cov, G));
-    return need <= (size_t)lim;
-  };
-  int ok = 0;
-  if (fits(4)) { e = setup_pot_g<R, 4>(cap_cov); ok |= 1; }
-  if (e == cudaSuccess && fits(8)) { e = setup_pot_g<R, 8>(cap_cov); ok |= 2; }
-  if (e == cudaSuccess) { e = setup_pot_g<R, 16>(cap_cov); ok |= 4; }
-  if (lanes_ok) *lanes_ok = ok;
+  bool f4 = false, f8 = false, f16 = false;
+  cudaError_t e = setup_pot_g<R, 4>(cap_cov, f4);
+  if (e == cudaSuccess) e = setup_pot_g<R, 8>(cap_cov, f8);
+  if (e == cudaSuccess) e = setup_pot_g<R, 16>(cap_cov, f16);
+  if (e == cudaSuccess && !f16) e = cudaErrorInvalidValue;
+  if (lanes_ok) *lanes_ok = (f4 ? 1 : 0) | (f8 ? 2 : 0) | (f16 ? 4 : 0);
   return e;
 }
 template cudaError_t setup_pot<float>(int, int*);
