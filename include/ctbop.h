@@ -113,7 +113,9 @@ typedef struct ctbop_params {
 
 typedef struct ctbop_options {
     int32_t precision;    /* CTBOP_PREC_FP64 or CTBOP_PREC_MIXED */
-    int32_t cg_max_iter;  /* charge-solve iteration cap (default 200) */
+    int32_t cg_max_iter;  /* charge-solve iteration cap (default 200); FP64 solves that refine in
+                             cycles (systems whose solve is one kernel): of each cycle, cg_iters_*
+                             counting all of them */
     double  cg_tol;       /* stop when max_i |H q + chi - mu|_i over a replica (the max-norm of
                            the stationarity residual) is below cg_tol (eV/e); 0 = policy default
                            (FP64 1e-11, MIXED 1e-5) */

@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
   // is a barrier of the block too):
   __shared__ double s_abc[2];   // alpha, beta: stored after the dots' exchange; c, mean: after that of y's sums
   __shared__ int s_stop;        // max |r - mean| met the goal: stored after the exchange of y's sums
-  __shared__ int s_fell;        // (FP64) the residual fell tenfold: stored after a cycle's first exchange of y's sums
+  __shared__ int s_fell;        // (FP64) the residual fell tenfold (1), a thousandfold (2): stored with a cycle's first s_stop
   __shared__ double s_shift;    // (FP64) the shift with the mean: stored after the CG of a cycle
   // (s_tot: stored by the exchanges between two of their own barriers, read by
   // any thread after an exchange and before it enters the next)
@@ -516,9 +516,14 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
         s_stop = key_of(bound) <= key_of(tol) ? 1 : 0;
       };
       // The CG in F from the residual ri (y = M^-1 r shared, its sums in
-      // s_abc), adding to dq, until max |r - mean| <= goal (the boss's) or
-      // the iterations are used up. Every block takes the same decisions.
-      int done = 0;
+      // s_abc), adding to dq, until max |r - mean| <= goal (the boss's; then
+      // `done`) or max_iter iterations are used up. The cap is that of one CG:
+      // the cycles of the FP64 policy each have it, because a CG that starts
+      // anew for every few digits takes more iterations in all than one that
+      // runs through (7 -> 11, 37 -> 44, 45 -> 50, 53 -> 55 from no charges), and
+      // what converged under a cap in one run has to converge under it here.
+      // Every block takes the same decisions.
+      int done = 1;
       auto iterate = [&](auto ri, auto yi, double goal, double& dq) -> bool {
         using F = decltype(ri);
         const F D = (F)Di, d = (F)di, v = (F)vi;
@@ -528,7 +533,7 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
         int stop = 0;
         const F* yb = reinterpret_cast<const F*>(yb1);
         const F* yg = reinterpret_cast<const F*>(A.y);
-        while (!stop && its < A.max_iter) {
+        for (int left = A.max_iter; !stop && left > 0; --left) {
           // ---- w = H z = H y - c v, z = y - c d, and the dots r.z, w.z
           if (unit) {
             PartSum<F> p0;
@@ -686,13 +691,15 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
             test(s_tot[0], s_tot[1], s_tot[2], s_tot[3], A.tol);
           }
           if constexpr (sizeof(R) == 8) {
-            s_fell = bound <= 0.1 * last ? 1 : 0;
+            s_fell = !(bound < INFINITY) ? 0 : bound <= 1e-3 * last ? 2 : bound <= 0.1 * last ? 1 : 0;
             last = bound;
           }
         }
         __syncthreads();
         conv = s_stop;
-        if (conv || its >= A.max_iter) break;   // (uniform: s_stop stays until the next exchange)
+        // (uniform: the words stay until the next exchange. At its cap short of
+        // its goal, a CG that gained three digits was stopped by FP32 rounding)
+        if (conv || (!done && s_fell < 2)) break;
         double dq = 0.0;
         bool go;
         if constexpr (sizeof(R) == 4) {
