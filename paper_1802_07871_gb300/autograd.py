@@ -19,9 +19,14 @@ class Energy(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x, system):
         xd = x.detach().to(torch.float64).contiguous()
+        ordered = x.is_cuda and system.ordered_with_current_stream()
+        if x.is_cuda and not ordered:
+            # what wrote the positions (their conversion among it) is in a
+            # stream that the system's does not wait for
+            torch.cuda.current_stream(x.device).synchronize()
         system.set_positions(xd.cpu().numpy() if not xd.is_cuda else xd)
         system.compute()
-        if x.is_cuda and system.ordered_with_current_stream():
+        if ordered:
             E = torch.empty(system.R, dtype=torch.float64, device=x.device)
             F = torch.empty((system.n, 3), dtype=torch.float64, device=x.device)
             system.get("energy", out=E)

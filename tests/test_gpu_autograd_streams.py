@@ -50,3 +50,36 @@ def test_energy_and_gradient_on_any_stream(where, dtype):
         assert np.max(np.abs(g + F)) <= tol * max(1.0, np.max(np.abs(F)))
     sysm.close()
     ref.close()
+
+
+@pytest.mark.parametrize("dtype", ["float32", "float64"])
+def test_positions_still_being_written_on_a_foreign_stream(dtype):
+    """The system does not know the stream that writes and converts the
+    positions: it has to wait for them all the same."""
+    import torch
+    from paper_1802_07871_gb300.autograd import Energy
+    s = st.sic_3c(2, 4.36, 0.05, seed=3)
+    ref = ctbop.System(P1, precision="fp64")
+    ref.load(s)
+    sysm = ctbop.System(P1, precision="fp64")
+    sysm.load(s)
+    dt = getattr(torch, dtype)
+    base = torch.tensor(s.x, dtype=dt, device="cuda")
+    x = base.clone().requires_grad_(True)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for k in range(2):
+        with torch.cuda.stream(stream):
+            torch.cuda._sleep(50_000_000)   # (some 25 ms before the positions are there)
+            with torch.no_grad():
+                x.copy_(base + 0.01 * (k + 1) * torch.sin(7.0 * base))
+            E = Energy.apply(x, sysm)
+            (g,) = torch.autograd.grad(E.sum(), x)
+        stream.synchronize()
+        ref.set_positions(x.detach().cpu().to(torch.float64).numpy())
+        ref.compute()
+        tol = 1e-8 if dtype == "float64" else 1e-6
+        assert np.max(np.abs(E.detach().cpu().numpy() - ref.get("energy"))) <= tol * abs(ref.get("energy")[0])
+        assert np.max(np.abs(g.cpu().numpy() + ref.get("forces"))) <= tol * max(1.0, np.max(np.abs(ref.get("forces"))))
+    sysm.close()
+    ref.close()
