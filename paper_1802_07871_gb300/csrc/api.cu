@@ -646,7 +646,10 @@ static int ensure_lists(ctbop_system* s) {
     int ca = cc + mc[1] + mc[1] / 8 + 16;
     cc = (cc + 3) & ~3;
     ca = (ca + 7) & ~7;
-    if (s->o.cap_cov > 0) cc = std::max(cc, s->o.cap_cov);
+    if (s->o.cap_cov > cc) {   // the rest comes after the places asked for
+      ca += s->o.cap_cov - cc;
+      cc = s->o.cap_cov;
+    }
     if (s->o.cap_all > 0) ca = std::max(ca, s->o.cap_all);
     if (over) {
       cc = std::max(cc, S.cap_cov);
