@@ -30,6 +30,7 @@
 // Sums are taken in a fixed order (lanes, warps, blocks), so a solve is
 // reproducible, and every block forms the same alpha, beta and decision.
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 #include <cooperative_groups.h>
 
@@ -831,6 +832,32 @@ cudaError_t launch_cg_solve(const DevState& S, const TypeParams& T, double tol, 
   return S.solver == SOLVE_CLUSTER ? launch_solve<R, true>(S, A, st) : launch_solve<R, false>(S, A, st);
 }
 
+// Whether a batch's clusters beat its launches, by an estimate of the time of an
+// iteration in microseconds. All clusters have the size that the largest
+// replica wants, `fit` of them run at a time (7 to 14 of 16 blocks), and a small
+// replica in a large cluster costs almost as much as a large one, its two
+// barriers; so the clusters take one wave of replicas after another, and the
+// launches their tails plus the stream of the matrix. Replicas of different size
+// also converge at different times: 0.6 of the iterations on average.
+// Measured, microseconds per MD step in clusters and by launches:
+//   mixed, even: 4, 12, 16, 24 x 8,000 atoms 362 and 502, 812 and 873, 1,152 and
+//   1,056, 1,630 and 1,426; 24, 48, 57 x 4,096 750 and 881, 1,454 and 1,499, 1,589
+//   and 1,556; 200 x 1,000 1,171 and 1,325; 1,000 x 64 433 and 618;
+//   mixed, uneven: 96 replicas of 200 to 3,000 atoms 1,360 and 1,507; 4,096 + 20 x 64
+//   209 and 375, + 100 x 64 392 and 388, + 1,000 x 64 2,884 and 782; 8,000 + 500 x 8
+//   1,500 and 422; 4,096 + 100 x 512 720 and 611; 1,728 + 500 x 64 425 and 471;
+//   FP64: 128 x 1,000 7,915 and 11,677; 4,096 + 100 x 64 2,770 and 2,776, + 1,000 x 64
+//   23,362 and 6,597; 1,728 + 500 x 64 3,621 and 4,089.
+static bool clusters_pay(bool fp32, int R, int N, double maxn, int size, int fit, int nsm, double row) {
+  const double mean = (double)N / R, some = maxn > 1.25 * mean ? 0.6 : 1.0;
+  const double barriers = 2.5 + 0.4 * size;
+  const double per_atom = 0.036 * std::max((double)fit * size / nsm, 1.0);   // of a block's share; blocks share an SM
+  const double waves = std::ceil((double)R / fit);
+  const double clusters = std::max(some * waves * (barriers + per_atom * mean / size), barriers + per_atom * maxn / size);
+  const double launches = (fp32 ? 35.0 : 66.0) + some * N * row / (fp32 ? 5.2e6 : 2.7e6);
+  return clusters < launches;
+}
+
 // Which form of the solve a system takes. The whole-solve kernel pays where
 // an iteration's time is its launches and tails; where it is the streaming
 // of a matrix larger than L2, the per-iteration kernels (every SM, whole
@@ -842,7 +869,8 @@ cudaError_t launch_cg_solve(const DevState& S, const TypeParams& T, double tol, 
 //     bandwidth and FP64 rate outweigh the cluster's cheaper barrier). Not
 //     past 3.5 L2 budgets of matrix in all: 96 replicas, 158,000 atoms take
 //     45 us per iteration in clusters against 55 by launches, 288 replicas,
-//     1.25 million atoms 0.57 ms against 0.33;
+//     1.25 million atoms 0.57 ms against 0.33. And not where clusters_pay
+//     says that the launches are faster;
 //   * one larger replica whose matrix fits L2: the grid-wide team;
 //   * anything else: the per-iteration kernels.
 // Solve times, microseconds per MD step by launches and with this kernel:
@@ -891,7 +919,8 @@ cudaError_t plan_cg_solve(DevState& S, const int64_t* off) {
     cfg.numAttrs = 1;
     int fit = 0;
     if (cfg.dynamicSmemBytes <= most_smem &&
-        cudaOccupancyMaxActiveClusters(&fit, k_cg_solve<R, true>, &cfg) == cudaSuccess && fit > 0) {
+        cudaOccupancyMaxActiveClusters(&fit, k_cg_solve<R, true>, &cfg) == cudaSuccess && fit > 0 &&
+        (!many || clusters_pay(sizeof(R) == 4, S.R, S.N, (double)maxn, size, fit, S.nsm, row))) {
       S.solver = SOLVE_CLUSTER;
       S.solve_blocks = size;
       S.solve_per = per;
