@@ -514,9 +514,17 @@ __global__ void __launch_bounds__(256)
 // 64 threads are no better.
 #define LG_T 128
 #define LG_B 4           // entries in flight per lane
-#define LG_FULL32 1300   // atoms per SM up to which FP32 takes 8 lanes per atom (at 158,391 atoms 173 + 153 us
-                         // against 190 + 205; at 1,005,466 atoms 2,410 + 1,183 against 938 + 970)
-#define LG_FULL64 2000   // the same for FP64 (its rows are bound by the FP64 pipe, not by their loads)
+// Atoms per SM up to which 8 lanes share an atom, else a thread each. FP32
+// assembly: two 256-atom tiles per SM (8 lanes and 1, microseconds: 41,616 atoms 66
+// and 94, 64,000 94 and 97, 85,184 121 and 117, 110,592 153 and 120, 129,650 174 and
+// 141, 195,112 297 and 227; just past a wave of tiles, at 158,000, 172 to 224 and 190
+// to 210). FP32 gather: 64,000 atoms 84 and 95, 110,592 130 and 129, 157,464 180 and
+// 233, 195,112 218 and 239, 216,000 241 and 240. FP64 (its rows are bound by the FP64
+// pipe, not by their loads): 18,928 atoms 457 and 1,044 (gather 175 and 1,530),
+// 110,592 2,609 and 3,193 (941 and 4,638), 296,208 6,901 and 8,486 (2,470 and 12,277).
+#define LG_ASM32 512
+#define LG_GATHER32 1300
+#define LG_FULL64 2000
 template <class R, int G>
 __global__ void __launch_bounds__(LG_T)
     k_assemble_g(int N, int cap_cov, int ld, const typename Vec4<R>::T* __restrict__ u,
@@ -1290,18 +1298,19 @@ void launch_bond(const DevState& S, const PotParams<R>& P, cudaStream_t st) {
   else launch_bond_g<R, 8>(S, P, st);
 }
 
-// Lanes per atom in the assembly and the charge-force gather: 1 (a thread
-// per atom, entries in flight per thread tuned) where that fills the chip,
-// else 8 or 32.
+// Lanes per atom in the assembly (gather false) and the charge-force gather: 1
+// (a thread per atom, entries in flight per thread tuned) where that fills the
+// chip, else 8 or 32. FP64 takes the same in both: the gather reads what the
+// assembly of several lanes keeps (S.kd).
 template <class R>
-static int row_lanes(const DevState& S) {
-  const int full = S.nsm * (sizeof(R) == 4 ? LG_FULL32 : LG_FULL64);
+static int row_lanes(const DevState& S, bool gather) {
+  const int full = S.nsm * (sizeof(R) == 8 ? LG_FULL64 : gather ? LG_GATHER32 : LG_ASM32);
   // (FP64 wants blocks of few atoms longer: rows of 70 to 240 entries in one
   // batch left the pipe 35% busy at 6,278 atoms with 32 atoms per block)
   return S.N <= S.nsm * (sizeof(R) == 4 ? 32 : 64) ? 32 : S.N <= full ? 8 : 1;
 }
 
-bool stored_kernel(const DevState& S) { return row_lanes<double>(S) > 1; }
+bool stored_kernel(const DevState& S) { return row_lanes<double>(S, true) > 1; }
 
 template <class R>
 void launch_assemble(const DevState& S, const PotParams<R>& P, const TypeParams& T, cudaStream_t st) {
@@ -1309,7 +1318,7 @@ void launch_assemble(const DevState& S, const PotParams<R>& P, const TypeParams&
 #define ASM_ARGS                                                                                        \
   S.N, S.cap_cov, S.ld, (const typename Vec4<R>::T*)S.u, S.rep, S.reps, S.nl, S.ncov, S.nfix, S.nall, S.rev, \
       (const typename Vec4<R>::T*)S.bo, P, T, S.M, (R*)S.Dg, (R*)S.dinv, S.nmat
-  const int g = (S.N + 255) / 256, lanes = row_lanes<R>(S), per = LG_T / lanes;
+  const int g = (S.N + 255) / 256, lanes = row_lanes<R>(S, false), per = LG_T / lanes;
   if (lanes == 32) k_assemble_g<R, 32><<<(S.N + per - 1) / per, LG_T, 0, st>>>(ASM_ARGS, S.kd);
   else if (lanes == 8) k_assemble_g<R, 8><<<(S.N + per - 1) / per, LG_T, 0, st>>>(ASM_ARGS, S.kd);
   else if (S.asm_batch == 4) k_assemble<R, 4><<<g, 256, 0, st>>>(ASM_ARGS);
@@ -1353,7 +1362,7 @@ template <class R>
 void launch_coul_gather(const DevState& S, const PotParams<R>& P, const TypeParams& T, int kick, double half_dt,
                         cudaStream_t st, bool virial, bool assembled) {
   if (S.N == 0) return;
-  const int lanes = row_lanes<R>(S);
+  const int lanes = row_lanes<R>(S, true);
   auto go = [&](auto kernel, auto... more) {
     int occ = 0, grid = 0;
     if (lanes > 1) {
