@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
   // is a barrier of the block too):
   __shared__ double s_abc[2];   // alpha, beta: stored after the dots' exchange; c, mean: after that of y's sums
   __shared__ int s_stop;        // max |r - mean| met the goal: stored after the exchange of y's sums
-  __shared__ int s_fell;        // (FP64) the residual fell tenfold (1), a thousandfold (2): stored with a cycle's first s_stop
+  __shared__ int s_fell;        // (FP64) the residual fell tenfold: stored with a cycle's first s_stop
   __shared__ double s_shift;    // (FP64) the shift with the mean: stored after the CG of a cycle
   // (s_tot: stored by the exchanges between two of their own barriers, read by
   // any thread after an exchange and before it enters the next)
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
   for (int rr = r_first; rr < r_end && alive; ++rr) {
     double* cc = A.cg + (size_t)rr * CG_STRIDE;
     const int a0 = A.reps[rr].atom_off, n = A.reps[rr].natoms;
-    int its = 0, conv = 0;
+    int its = 0, total = 0, conv = 0;   // iterations of this CG, of the ones before it
     if (n == 0) {
       if (T.rank == 0 && threadIdx.x == 0) cc[CG_RESMAX] = cc[CG_RES0] = INFINITY;
       conv = 1;
@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
         int stop = 0;
         const F* yb = reinterpret_cast<const F*>(yb1);
         const F* yg = reinterpret_cast<const F*>(A.y);
-        for (int left = A.max_iter; !stop && left > 0; --left) {
+        while (!stop && its < A.max_iter) {
           // ---- w = H z = H y - c v, z = y - c d, and the dots r.z, w.z
           if (unit) {
             PartSum<F> p0;
@@ -625,7 +625,7 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
       // nearer the minimiser than by the recursion's residual). Should a cycle gain less than a
       // digit, the CG goes on in FP64, to the tolerance by its own recursion (a
       // tolerance at the FP64 residual's rounding can be met that way only).
-      double last = INFINITY;
+      double last = 1e308;
       bool final_shift = false;
       for (int cycle = 0;; ++cycle) {
         if (in) share(yb0, A.qr, (R)qi);
@@ -692,17 +692,18 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
             test(s_tot[0], s_tot[1], s_tot[2], s_tot[3], A.tol);
           }
           if constexpr (sizeof(R) == 8) {
-            s_fell = !(bound < INFINITY) ? 0 : bound <= 1e-3 * last ? 2 : bound <= 0.1 * last ? 1 : 0;
+            s_fell = bound <= 0.1 * last ? 1 : 0;   // (0 if it is not finite)
             last = bound;
           }
         }
         __syncthreads();
         conv = s_stop;
-        // (uniform: the words stay until the next exchange. At its cap short of
-        // its goal, a CG that gained three digits was stopped by FP32 rounding)
-        if (conv || (!done && s_fell < 2)) break;
+        // (uniform: the word stays until the next exchange)
+        if (conv || !done) break;
         double dq = 0.0;
         bool go;
+        total += its;
+        its = 0;
         if constexpr (sizeof(R) == 4) {
           go = iterate(ri, yf, A.tol, dq);
           qi += dq;
@@ -760,6 +761,7 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
       }
     }
     if (T.rank == 0 && threadIdx.x == 0) {
+      its += total;   // all of them
       A.conv[rr] = conv;
       A.iters[rr] = its;
       if (!conv) atomicOr(A.err, CT_ERR_CG_MAXITER);
