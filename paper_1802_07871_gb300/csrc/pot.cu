@@ -514,16 +514,21 @@ __global__ void __launch_bounds__(256)
 // 64 threads are no better.
 #define LG_T 128
 #define LG_B 4           // entries in flight per lane
-// Atoms per SM up to which 8 lanes share an atom, else a thread each. FP32
-// assembly: two 256-atom tiles per SM (8 lanes and 1, microseconds: 41,616 atoms 66
-// and 94, 64,000 94 and 97, 85,184 121 and 117, 110,592 153 and 120, 129,650 174 and
-// 141, 195,112 297 and 227; just past a wave of tiles, at 158,000, 172 to 224 and 190
-// to 210). FP32 gather: 64,000 atoms 84 and 95, 110,592 130 and 129, 157,464 180 and
-// 233, 195,112 218 and 239, 216,000 241 and 240. FP64 (its rows are bound by the FP64
-// pipe, not by their loads): 18,928 atoms 457 and 1,044 (gather 175 and 1,530),
-// 110,592 2,609 and 3,193 (941 and 4,638), 296,208 6,901 and 8,486 (2,470 and 12,277).
-#define LG_ASM32 512
+// Up to what 8 lanes share an atom, else a thread each.
+// FP32 assembly: where a thread per atom leaves its waves of four 256-atom tiles
+// per SM at most about half full, which is up to about two tiles per SM (80,896 atoms) and
+// just past a wave (155,649 to 161,792). 8 lanes and 1, microseconds: 41,616 atoms 66 and 94,
+// 64,000 94 and 97; 85,184 121 and 117, 110,592 153 and 120, 129,650 174 and 141;
+// 157,464 to 162,110 atoms 224 and 210, 219 and 222, 174 and 188 (uneven rows);
+// 195,112 297 and 227, 216,000 337 and 244.
+#define LG_ASM_TILES 4
+#define LG_ASM_FULL 0.52
+// FP32 gather (its grid strides over the tiles): atoms per SM. 64,000 atoms 84 and
+// 95, 110,592 130 and 129, 157,464 180 and 233, 195,112 218 and 239, 216,000 241 and 240.
 #define LG_GATHER32 1300
+// FP64, both (rows bound by the FP64 pipe, not by their loads): 18,928 atoms 457 and
+// 1,044 (gather 175 and 1,530), 110,592 2,609 and 3,193 (941 and 4,638), 296,208 6,901
+// and 8,486 (2,470 and 12,277).
 #define LG_FULL64 2000
 template <class R, int G>
 __global__ void __launch_bounds__(LG_T)
@@ -1304,10 +1309,14 @@ void launch_bond(const DevState& S, const PotParams<R>& P, cudaStream_t st) {
 // assembly of several lanes keeps (S.kd).
 template <class R>
 static int row_lanes(const DevState& S, bool gather) {
-  const int full = S.nsm * (sizeof(R) == 8 ? LG_FULL64 : gather ? LG_GATHER32 : LG_ASM32);
+  bool full = S.N > S.nsm * (sizeof(R) == 8 ? LG_FULL64 : LG_GATHER32);
+  if (sizeof(R) == 4 && !gather) {
+    const int tiles = (S.N + 255) / 256, wave = LG_ASM_TILES * S.nsm;
+    full = tiles > LG_ASM_FULL * ((tiles + wave - 1) / wave * wave);
+  }
   // (FP64 wants blocks of few atoms longer: rows of 70 to 240 entries in one
   // batch left the pipe 35% busy at 6,278 atoms with 32 atoms per block)
-  return S.N <= S.nsm * (sizeof(R) == 4 ? 32 : 64) ? 32 : S.N <= full ? 8 : 1;
+  return S.N <= S.nsm * (sizeof(R) == 4 ? 32 : 64) ? 32 : full ? 1 : 8;
 }
 
 bool stored_kernel(const DevState& S) { return row_lanes<double>(S, true) > 1; }

@@ -1,5 +1,5 @@
 """The FP32 assembly and charge-force gather on either side of the lines between
-8 lanes and a thread per atom (512 and 1,300 atoms per SM): small replicas
+8 lanes and a thread per atom (80,896 and 197,600 atoms): small replicas
 alone and in batches between the lines and above both."""
 import numpy as np
 import pytest
