@@ -1872,8 +1872,8 @@ int ctbop_rings(ctbop_system* s, double bond_cut, int32_t max_size, int64_t cap,
   unsigned long long* d_cnt = nullptr;
   Scratch scr(s->stream, s->pool);
   CK(scr.alloc(&d_out, (size_t)std::max<int64_t>(cap, 1)));
-  CK(scr.alloc(&d_cnt, 2));
-  CK(zero_async(s, d_cnt, 2 * sizeof(unsigned long long)));
+  CK(scr.alloc(&d_cnt, 3));
+  CK(zero_async(s, d_cnt, 3 * sizeof(unsigned long long)));
   CK(s->mixed ? launch_rings<float>(s->S, bond_cut, max_size, d_out, cap, d_cnt, s->stream)
               : launch_rings<double>(s->S, bond_cut, max_size, d_out, cap, d_cnt, s->stream));
   unsigned long long got[2] = {0, 0};

@@ -272,7 +272,8 @@ template <class R>
 void launch_fire_move(const DevState& S, const TypeParams& T, const double* fire, double half_skin2,
                       cudaStream_t st);
 // Primitive C rings (csrc/rings.cu): records appended through count[0] (the
-// total, which may exceed cap; records past cap are dropped). count[1] atoms
+// total, which may exceed cap; records past cap are dropped); count[0..2] are
+// zero before. count[1] atoms
 // are left over: launch_rings_wide searches them (pass 0, 1, ...) with tables
 // of `slots` places (a power of two) in rings_wide_bytes of device memory, and
 // leaves in count[1], cleared before, those that want larger ones.

@@ -27,6 +27,7 @@
 // per atom, through the strided lists, took 151 ms on 96 replicas (158,391
 // atoms) where a call now takes 3.0 ms.
 #include <math.h>
+#include <algorithm>
 
 #include "ctbop.h"
 #include "internal.cuh"
@@ -46,7 +47,8 @@ __device__ inline int bits_int(float x) { return __float_as_int(x); }
 __device__ inline int bits_int(double x) { return (int)__double_as_longlong(x); }
 
 // The C-C bonds of every C atom: entry k of atom v at v * cap + k, the bond
-// vector and (bits of w) the partner.
+// vector and (bits of w) the partner; and the atoms with two or more, which are
+// the ones to search.
 template <class R>
 struct RingGraph {
   typename Vec4<R>::T* bond;
@@ -58,11 +60,13 @@ template <class R>
 __global__ void k_ring_graph(int N, int ld, int cap, const typename Vec4<R>::T* __restrict__ u,
                              const int* __restrict__ rep, const RepInfo* __restrict__ reps,
                              const int2* __restrict__ nl, const int* __restrict__ ncov, R cut2,
-                             typename Vec4<R>::T* __restrict__ bond, int* __restrict__ deg) {
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= N) return;
-  const typename Vec4<R>::T uv = u[v];
+                             typename Vec4<R>::T* __restrict__ bond, int* __restrict__ deg, int* __restrict__ cand,
+                             unsigned long long* __restrict__ n_cand) {
+  const int v = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
   int n = 0;
+  typename Vec4<R>::T uv;
+  uv.w = R(0);
+  if (v < N) uv = u[v];
   if ((int)uv.w == 1) {
     const RepInfo& ri = reps[rep[v]];
     R hx = ri.hcf[0], hy = ri.hcf[1], hz = ri.hcf[2];
@@ -84,7 +88,14 @@ __global__ void k_ring_graph(int N, int ld, int cap, const typename Vec4<R>::T* 
       ++n;
     }
   }
-  deg[v] = n;
+  if (v < N) deg[v] = n;
+  const bool c = n >= 2;   // (no ring closes through one bond)
+  const unsigned m = __ballot_sync(CT_FULL, c);
+  if (m == 0u) return;
+  int at = 0;
+  if (lane == 0) at = (int)atomicAdd(n_cand, (unsigned long long)__popc(m));
+  at = __shfl_sync(CT_FULL, at, 0);
+  if (c) cand[at + __popc(m & ((1u << lane) - 1u))] = v;
 }
 
 template <class R>
@@ -203,7 +214,6 @@ __device__ bool ring_search(int a, const RingTable<R>& T, const RingGraph<R>& G,
   const unsigned lt = (1u << lane) - 1u;
   const int most = T.slots * 3 / 4;
   const int da = G.deg[a];
-  if (da < 2) return true;   // (no ring closes through one bond)
   // ---- 1. breadth first
   for (int k = lane; k < T.slots; k += 32) T.key[k] = -1;
   __syncwarp();
@@ -322,17 +332,20 @@ __device__ bool ring_search(int a, const RingTable<R>& T, const RingGraph<R>& G,
 
 template <class R>
 __global__ void __launch_bounds__(RING_WARPS * 32)
-    k_rings(int N, RingGraph<R> G, const double* __restrict__ x, const int* __restrict__ rep, int max_size,
-            ctbop_ring* __restrict__ out, long long cap, unsigned long long* __restrict__ count,
+    k_rings(const int* __restrict__ cand, RingGraph<R> G, const double* __restrict__ x, const int* __restrict__ rep,
+            int max_size, ctbop_ring* __restrict__ out, long long cap, unsigned long long* __restrict__ count,
             int* __restrict__ wide) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   RingTable<R> T;
   T.place(smem_raw + warp * RingTable<R>::bytes(RING_SLOTS), RING_SLOTS);
-  const int a = blockIdx.x * RING_WARPS + warp;
-  if (a >= N) return;
-  if (!ring_search(a, T, G, x, rep, max_size, out, cap, count) && (threadIdx.x & 31) == 0)
-    wide[atomicAdd(count + 1, 1ull)] = a;
+  const int n = (int)count[2];
+  // (neighbours of the list to one block: they share bonds in L1)
+  for (int t = blockIdx.x * RING_WARPS + warp; t < n; t += gridDim.x * RING_WARPS) {
+    const int a = cand[t];
+    if (!ring_search(a, T, G, x, rep, max_size, out, cap, count) && lane == 0) wide[atomicAdd(count + 1, 1ull)] = a;
+    __syncwarp();
+  }
 }
 
 // The queued atoms, with a table of `slots` in global memory for each warp
@@ -356,7 +369,16 @@ __global__ void __launch_bounds__(RING_WARPS * 32)
 
 // Scratch of the search, per atom: the bonds in the force slots (Real4 per
 // covalent entry; every force pass writes its slots before it reads them), the
-// degrees and the two queues in the staging buffer (24 bytes an atom).
+// degrees, the two queues and the list of atoms to search in the staging buffer
+// (16 of its 24 bytes an atom).
+//
+// The grid is at most eight times what is resident at once, and strides over the
+// listed atoms: a warp per atom of the system, none with anything to do in SiC,
+// took 89 us a call on a slab of 397,490 atoms without C-C bonds, where an
+// exhaustive search's threads had taken 44; this 42. (The resident blocks alone, or
+// warps that fetch one atom after another, lose 3 to 7% where C abounds: uneven
+// shares, and neighbours spread over the SMs.) The ensemble of 158,391 atoms
+// 2,480 -> 2,145 us, a graphene sheet of 20,088 atoms 444 -> 465.
 template <class R>
 cudaError_t launch_rings(const DevState& S, double bond_cut, int max_size, ctbop_ring* out, long long cap,
                          unsigned long long* count, cudaStream_t st) {
@@ -364,9 +386,15 @@ cudaError_t launch_rings(const DevState& S, double bond_cut, int max_size, ctbop
   int* deg = static_cast<int*>(S.stage);
   RingGraph<R> G{(typename Vec4<R>::T*)S.gslot, deg, S.cap_cov};
   k_ring_graph<R><<<(S.N + 255) / 256, 256, 0, st>>>(S.N, S.ld, S.cap_cov, (const typename Vec4<R>::T*)S.u, S.rep,
-                                                     S.reps, S.nl, S.ncov, (R)(bond_cut * bond_cut), G.bond, deg);
-  k_rings<R><<<(S.N + RING_WARPS - 1) / RING_WARPS, RING_WARPS * 32, RING_WARPS * RingTable<R>::bytes(RING_SLOTS), st>>>(
-      S.N, G, S.x, S.rep, max_size, out, cap, count, deg + S.N);
+                                                     S.reps, S.nl, S.ncov, (R)(bond_cut * bond_cut), G.bond, deg,
+                                                     deg + (size_t)3 * S.N, count + 2);
+  const size_t smem = RING_WARPS * RingTable<R>::bytes(RING_SLOTS);
+  int occ = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_rings<R>, RING_WARPS * 32, smem);
+  if (e != cudaSuccess) return e;
+  const int grid = std::min((S.N + RING_WARPS - 1) / RING_WARPS, 8 * S.nsm * std::max(occ, 1));
+  k_rings<R><<<grid, RING_WARPS * 32, smem, st>>>(deg + (size_t)3 * S.N, G, S.x, S.rep, max_size, out, cap, count,
+                                                  deg + S.N);
   return cudaGetLastError();
 }
 
