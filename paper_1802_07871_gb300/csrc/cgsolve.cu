@@ -16,10 +16,9 @@
 //     barrier, partial sums exchanged through distributed shared memory, and
 //     every block holding the replica's whole y, which the others write into
 //     its shared memory. Replicas converge and leave on their own.
-//   * all blocks of a cooperative launch on one replica after another: y
-//     and the partial sums in global memory, a counter as the barrier
-//     (cooperative, so every block is resident; the wait is bounded all the
-//     same).
+//   * all blocks of a cooperative launch on a lone replica: y and the partial
+//     sums in global memory, a counter as the barrier (cooperative, so every
+//     block is resident; the wait is bounded all the same).
 //
 // Layout: a block owns up to CS_W groups of 32 consecutive atoms (the
 // preconditioner's blocks). Warp g of it holds group g's vectors (r, p, s,
@@ -356,10 +355,10 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
   constexpr int NCH = BlockChunk<R>::NCH;
   R* yb0 = reinterpret_cast<R*>(s_blk + (A.binv ? (size_t)A.per * NCH * 32 : 0));   // cluster team: the replica's q,
   R* yb1 = yb0 + A.maxn;                               // and its y, both written by every block of the cluster
-  const int r_first = CL ? (int)(blockIdx.x / T.size) : 0, r_end = CL ? r_first + 1 : A.Rn;
+  const int rr = CL ? (int)(blockIdx.x / T.size) : 0;
   const int nh = *A.hist;
   bool alive = true;
-  for (int rr = r_first; rr < r_end && alive; ++rr) {
+  do {   // (once: left early when a wait gave up)
     double* cc = A.cg + (size_t)rr * CG_STRIDE;
     const int a0 = A.reps[rr].atom_off, n = A.reps[rr].natoms;
     int its = 0, total = 0, conv = 0;   // iterations of this CG, of the ones before it
@@ -777,7 +776,7 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
         *A.hist = h < 3 ? h + 1 : 3;
       }
     }
-  }
+  } while (false);
   if constexpr (!CL) {   // the last block to leave clears the counter for the next solve
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -871,8 +870,11 @@ static bool clusters_pay(bool fp32, int R, int N, double maxn, int size, int fit
 //     bandwidth and FP64 rate outweigh the cluster's cheaper barrier). Not
 //     past 3.5 L2 budgets of matrix in all: 96 replicas, 158,000 atoms take
 //     45 us per iteration in clusters against 55 by launches, 288 replicas,
-//     1.25 million atoms 0.57 ms against 0.33. And not where clusters_pay
-//     says that the launches are faster;
+//     1.25 million atoms 0.57 ms against 0.33 (past the line clusters still
+//     win with small replicas, 500 x 512 atoms 1,276 us per step against
+//     1,557, 4,000 x 64 1,386 against 1,809, and lose with large ones, 72 x
+//     4,096 2,011 against 1,903). And not where clusters_pay says that the
+//     launches are faster;
 //   * one larger replica whose matrix fits L2: the grid-wide team;
 //   * anything else: the per-iteration kernels.
 // Solve times, microseconds per MD step by launches and with this kernel:

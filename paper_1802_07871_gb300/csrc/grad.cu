@@ -81,8 +81,6 @@ __device__ inline double flog(double x) { return log(x); }
 __device__ inline float flog(float x) { return logf(x); }
 __device__ inline double fpow(double x, double n) { return pow(x, n); }
 __device__ inline float fpow(float x, float n) { return powf(x, n); }
-__device__ inline double fcbrt(double x) { return cbrt(x); }
-__device__ inline float fcbrt(float x) { return cbrtf(x); }
 __device__ inline double fcospi(double x) { return cospi(x); }
 __device__ inline float fcospi(float x) { return cospif(x); }
 __device__ inline double fsinpi(double x) { return sinpi(x); }
@@ -92,10 +90,6 @@ template <class T> __device__ inline DualT<T> flog(DualT<T> x) { return {flog(x.
 template <class T> __device__ inline DualT<T> fpow(DualT<T> x, T n) {   // x.v > 0
   T p = fpow(x.v, n);
   return {p, n * p * inv(x.v) * x.d};
-}
-template <class T> __device__ inline DualT<T> fcbrt(DualT<T> x) {
-  T c = fcbrt(x.v);
-  return {c, x.d / (T(3) * c * c)};
 }
 template <class T> __device__ inline DualT<T> fcospi(DualT<T> x) {
   return {fcospi(x.v), -T(M_PI) * fsinpi(x.v) * x.d};
@@ -491,7 +485,8 @@ __global__ void __launch_bounds__(NT)
 // the three the sums' tangents follow; vout_i gets the Coulomb share of
 // d(Hq + chi)_i/de, ke sum_j q_j k' tr. QDIR: the charges carry theirs. (The
 // general dual numbers with a power, a cube root and six divisions per entry,
-// one thread per atom, took 6.5 ms in FP64 on 6,278 atoms; this 0.15.)
+// one thread per atom, took 6.5 ms in FP64 on 6,278 atoms; this 0.39 along dir,
+// 0.28 along q.)
 #define PC_T 256
 #define PC_G 8
 template <class R, bool DIR, bool QDIR>

@@ -130,7 +130,7 @@ struct DevState {
   int* flag_rebuild = nullptr;
   int* flag_one = nullptr;      // a flag that stays 1 (list-build tuning)
   long long* rebuild_count = nullptr;
-  int* maxcnt = nullptr;        // [3] at the last rebuild: max ncov, max count of the rest, max nall
+  int* maxcnt = nullptr;        // [4] at the last rebuild: max ncov, max count of the rest, max nall; then the error word
   unsigned* err = nullptr;
   int* cg_it = nullptr;         // iteration counter of the running solve
   int* cg_blocks = nullptr;     // last-block counters [3]

@@ -1115,7 +1115,10 @@ __global__ void __launch_bounds__(LG_T)
       if (sizeof(R) == 4) {
 #pragma unroll
         for (int k = 0; k < LG_B; ++k) ec.add(en[k]);
-      } else {   // (FP64: the batch first, then one compensated addition)
+      } else {
+        // (FP64: the batch first, then one compensated addition. The per-atom
+        // energies of 13,824 atoms are as far from extended precision as with an
+        // addition each, 2.58e-15 eV rms, for 175 instead of 217 us at 18,928 atoms)
         ec.add((en[0] + en[1]) + (en[2] + en[3]));
       }
     }
@@ -1603,7 +1606,8 @@ template cudaError_t tune_cov<double>(DevState&, const PotParams<double>&, const
 // state of a completed evaluation without a kick, each depth runs the
 // covalent force pass (untimed: the gather adds to the per-atom energies it
 // writes) and the gather without the virial (timed: the variant MD steps
-// run), three times; the fastest is kept and the pair runs once more, with
+// run; where several lanes share an atom, see row_lanes, the depth is not used
+// and the three timings are of one kernel), three times; the fastest is kept and the pair runs once more, with
 // the virial, so the evaluation's results are as the kept depth sums them.
 template <class R>
 cudaError_t tune_gather(DevState& S, const PotParams<R>& P, const TypeParams& T, cudaStream_t st, float* ms_out) {

@@ -66,6 +66,10 @@ def _parse(t, lambdas):
             e = _close(t, b)
             lambdas[m.group(1)] = _parse(t[b + 1:e - 1], lambdas)
             i = e + 1
+        elif m := re.compile(r"do\s*(?=\{)").match(t, i):   # (once)
+            e = _close(t, m.end())
+            out += _parse(t[m.end() + 1:e - 1], lambdas)
+            i = t.index(";", e) + 1
         elif t[i] == "{":
             e = _close(t, i)
             out += _parse(t[i + 1:e - 1], lambdas)
