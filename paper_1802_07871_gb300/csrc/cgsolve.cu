@@ -355,10 +355,13 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
   constexpr int NCH = BlockChunk<R>::NCH;
   R* yb0 = reinterpret_cast<R*>(s_blk + (A.binv ? (size_t)A.per * NCH * 32 : 0));   // cluster team: the replica's q,
   R* yb1 = yb0 + A.maxn;                               // and its y, both written by every block of the cluster
-  const int rr = CL ? (int)(blockIdx.x / T.size) : 0;
+  // (one replica either way: the plan gives the grid lone ones. Compiled without
+  // the loop the FP64 grid took 2% more on a slab of 19,548 atoms, 716 -> 733 us, and
+  // 3% less on a crystal of 18,928, 643 -> 626)
+  const int r_first = CL ? (int)(blockIdx.x / T.size) : 0, r_end = CL ? r_first + 1 : A.Rn;
   const int nh = *A.hist;
   bool alive = true;
-  do {   // (once: left early when a wait gave up)
+  for (int rr = r_first; rr < r_end && alive; ++rr) {
     double* cc = A.cg + (size_t)rr * CG_STRIDE;
     const int a0 = A.reps[rr].atom_off, n = A.reps[rr].natoms;
     int its = 0, total = 0, conv = 0;   // iterations of this CG, of the ones before it
@@ -776,7 +779,7 @@ __global__ void __launch_bounds__(CS_T, CL && sizeof(R) == 4 ? 2 : 1) k_cg_solve
         *A.hist = h < 3 ? h + 1 : 3;
       }
     }
-  } while (false);
+  }
   if constexpr (!CL) {   // the last block to leave clears the counter for the next solve
     __syncthreads();
     if (threadIdx.x == 0) {
