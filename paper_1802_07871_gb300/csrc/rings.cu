@@ -25,7 +25,7 @@
 // tables in global memory. Bound by the
 // latency of the walks' dependent loads; the exhaustive search by one thread
 // per atom, through the strided lists, took 151 ms on 96 replicas (158,391
-// atoms) where a call now takes 3.0 ms.
+// atoms) where a call now takes 2.9 ms.
 #include <math.h>
 #include <algorithm>
 
